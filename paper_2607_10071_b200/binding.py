@@ -1,8 +1,10 @@
-"""Thin ctypes binding of the C ABI in include/flashbev.h.
+"""Thin binding of the C ABI in include/flashbev.h.
 
 Argument marshalling only: every step of the operator runs inside the CUDA
-library.  PyTorch is used by callers for device memory and streams; this module
-needs only integer addresses.  There is no CPU fallback: if the library has not
+library.  PyTorch is used by callers for device memory and streams; the ctypes
+part of this module needs only integer addresses, the functions for torch
+tensors (``sampling_vt`` and the like) marshal in the extension module
+``_native`` (csrc/native.cpp).  There is no CPU fallback: if the library has not
 been built, or the call fails, an exception is raised.
 """
 from __future__ import annotations
@@ -160,6 +162,30 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native = None
+
+
+def native():
+    """The extension module over libflashbev.so (built in-tree by ``paper_2607_10071_b200.build``)."""
+    global _native
+    if _native is None:
+        import torch  # noqa: F401  (its libraries have to be loaded first)
+        try:
+            from . import _native as module
+        except ImportError as e:
+            raise ImportError("the extension module is missing: build it with `python -m paper_2607_10071_b200.build` "
+                              "(there is no CPU fallback)") from e
+        _native = module
+    return _native
+
+
+def _result(r, what):
+    """A result tensor of the extension module, or the status of a refused call raised."""
+    if type(r) is int:
+        raise FlashBevError(r, what)
+    return r
+
+
 def status_string(status: int) -> str:
     return lib().flashbev_status_string(int(status)).decode()
 
@@ -267,21 +293,8 @@ def flashbev_sampling_vt_backward(params: VtBackwardParams, stream: int | None =
 def sampling_vt_backward(grad_out, lidar2img, feat_hw, img_hw, bev_range, grid, reduce=REDUCE_SUM,
                          grad_features=None, tune=(0, 0, 0, 0), stream=None):
     """grad_out: CUDA float32 [B,X,Y,C]; returns CUDA float32 [B,N,Hf,Wf,C] (marshalling only)."""
-    import torch
-
-    if not grad_out.is_cuda or grad_out.dtype != torch.float32 or not grad_out.is_contiguous():
-        raise ValueError("grad_out must be a contiguous CUDA float32 tensor")
-    B, X, Y, C = grad_out.shape
-    N = lidar2img.shape[1]
-    if grad_features is None:
-        grad_features = torch.empty((B, N, feat_hw[0], feat_hw[1], C), dtype=torch.float32, device=grad_out.device)
-    p = make_backward_params(grad_out.data_ptr(), lidar2img.data_ptr(), B, N, C, feat_hw, img_hw, bev_range,
-                             (X, Y, grid[2]), reduce, grad_features.data_ptr(), tune)
-    if stream is None:
-        stream = torch.cuda.current_stream(grad_out.device).cuda_stream
-    with torch.cuda.device(grad_out.device):
-        flashbev_sampling_vt_backward(p, stream)
-    return grad_features
+    return _result((_native or native()).sampling_vt_backward(grad_out, lidar2img, feat_hw, img_hw, bev_range, grid, reduce,
+                                                              grad_features, tune, stream), "flashbev_sampling_vt_backward")
 
 
 def flashbev_sca(params: ScaParams, stream: int | None = None, check: bool = True) -> int:
@@ -296,37 +309,8 @@ def sca(value, level_hw, lidar2img, offsets, weights, img_hw, bev_range, grid, o
         chunk_records=0):
     """value: CUDA float32 or bfloat16 [B,N,T,heads,Dh]; offsets [B,Q,heads,L,P,2]; weights [B,Q,heads,L,P] (CUDA float32).
     level_hw: sequence of (H_l, W_l).  Returns CUDA float32 [B, Q, heads*Dh] (marshalling only)."""
-    import numpy as np
-    import torch
-
-    for t in (lidar2img, offsets, weights):
-        if not t.is_cuda or t.dtype != torch.float32 or not t.is_contiguous():
-            raise ValueError("sca needs contiguous CUDA float32 tensors")
-    if not value.is_cuda or not value.is_contiguous() or value.dtype not in (torch.float32, torch.bfloat16):
-        raise ValueError("value must be a contiguous CUDA float32 or bfloat16 tensor")
-    B, N, T, heads, Dh = value.shape
-    X, Y, Zref = grid
-    L, P = weights.shape[3], weights.shape[4]
-    lv = np.ascontiguousarray(level_hw, np.int32)
-    if out is None:
-        out = torch.empty((B, X * Y, heads * Dh), dtype=torch.float32, device=value.device)
-    p = ScaParams()
-    p.struct_size = ctypes.sizeof(ScaParams)
-    p.value, p.chunk_records = value.data_ptr(), int(chunk_records)
-    p.value_dtype = F32 if value.dtype == torch.float32 else BF16
-    p.level_hw = lv.ctypes.data
-    p.lidar2img, p.offsets, p.weights = lidar2img.data_ptr(), offsets.data_ptr(), weights.data_ptr()
-    p.B, p.N, p.heads, p.head_dim, p.L, p.P = B, N, heads, Dh, L, P
-    p.img_h, p.img_w = img_hw
-    p.x_min, p.x_max, p.y_min, p.y_max, p.z_min, p.z_max = (float(v) for v in bev_range)
-    p.X, p.Y, p.Zref = X, Y, Zref
-    p.out = out.data_ptr()
-    p.hits_out = None if hits is None else hits.data_ptr()
-    if stream is None:
-        stream = torch.cuda.current_stream(value.device).cuda_stream
-    with torch.cuda.device(value.device):
-        flashbev_sca(p, stream)
-    return out
+    return _result((_native or native()).sca(value, level_hw, lidar2img, offsets, weights, img_hw, bev_range, grid, out, hits,
+                                             stream, chunk_records), "flashbev_sca")
 
 
 def flashbev_workspace_bytes(params: VtParams) -> int:
@@ -357,84 +341,14 @@ def sampling_vt(features, lidar2img, img_hw, bev_range, grid, reduce=REDUCE_SUM,
     ``workspace``: for NCHW tensors and for channel counts that are not whole 16-byte vectors, lend the call the
     scratch ``flashbev_workspace_bytes`` asks for (a torch allocation, or a uint8 CUDA tensor of the caller's);
     False: none, the generic kernel runs."""
-    import torch
-
-    if not features.is_cuda or not lidar2img.is_cuda:
-        raise ValueError("sampling_vt needs CUDA tensors; there is no CPU path")
-    if not features.is_contiguous() or not lidar2img.is_contiguous():
-        raise ValueError("features and lidar2img must be contiguous")
-    if features.dtype == torch.float32:
-        dt = F32
-    elif features.dtype == torch.bfloat16:
-        dt = BF16
-    else:
-        raise ValueError("features must be float32 or bfloat16")
-    if lidar2img.dtype != torch.float32:
-        raise ValueError("lidar2img must be float32")
-    if layout == NHWC:
-        B, N, Hf, Wf, C = features.shape
-    else:
-        B, N, C, Hf, Wf = features.shape
-    X, Y, Z = grid
-    if out is None:
-        out = torch.empty((B, X, Y, C) if layout == NHWC else (B, C, X, Y),
-                          dtype=torch.float32 if out_dtype == F32 else torch.bfloat16, device=features.device)
-    p = make_params(features.data_ptr(), dt, lidar2img.data_ptr(), B, N, C, (Hf, Wf), img_hw, bev_range,
-                    (X, Y, Z), reduce, out.data_ptr(),
-                    None if valid_count is None else valid_count.data_ptr(), kernel, tune, layout, out_dtype)
-    if workspace is not False and workspace is not None:
-        need = flashbev_workspace_bytes(p)
-        if need:
-            ws = workspace if workspace is not True else torch.empty(need, dtype=torch.uint8, device=features.device)
-            p.workspace, p.workspace_bytes = ws.data_ptr(), ws.numel() * ws.element_size()
-    if stream is None:
-        stream = torch.cuda.current_stream(features.device).cuda_stream
-    with torch.cuda.device(features.device):
-        flashbev_sampling_vt(p, stream)
-    return out
+    return _result((_native or native()).sampling_vt(features, lidar2img, img_hw, bev_range, grid, reduce, out, valid_count,
+                                                     kernel, tune, stream, layout, out_dtype, workspace), "flashbev_sampling_vt")
 
 
 def sampling_vt_multires(features, lidar2img, img_hw, bev_range, grid, reduce=REDUCE_SUM, out=None,
                          valid_count=None, kernel=KERNEL_AUTO, tune=(0, 0, 0, 0), stream=None, layout=NHWC):
     """features: sequence of CUDA tensors, one per pyramid level, each [B,N,Hf_l,Wf_l,C] (NHWC) or
     [B,N,C,Hf_l,Wf_l] (NCHW) of one dtype.  Returns the float32 sum over the levels (marshalling only)."""
-    import torch
-
-    f0 = features[0]
-    for f in features:
-        if not f.is_cuda or not f.is_contiguous() or f.dtype != f0.dtype:
-            raise ValueError("every level must be a contiguous CUDA tensor of the same dtype")
-    if f0.dtype == torch.float32:
-        dt = F32
-    elif f0.dtype == torch.bfloat16:
-        dt = BF16
-    else:
-        raise ValueError("features must be float32 or bfloat16")
-    if not lidar2img.is_cuda or lidar2img.dtype != torch.float32 or not lidar2img.is_contiguous():
-        raise ValueError("lidar2img must be a contiguous CUDA float32 tensor")
-    if layout == NHWC:
-        B, N, _, _, C = f0.shape
-        hws = [(f.shape[2], f.shape[3]) for f in features]
-    else:
-        B, N, C, _, _ = f0.shape
-        hws = [(f.shape[3], f.shape[4]) for f in features]
-    X, Y, Z = grid
-    if out is None:
-        out = torch.empty((B, X, Y, C) if layout == NHWC else (B, C, X, Y), dtype=torch.float32, device=f0.device)
-    base = make_params(f0.data_ptr(), dt, lidar2img.data_ptr(), B, N, C, hws[0], img_hw, bev_range, (X, Y, Z),
-                       reduce, out.data_ptr(), None if valid_count is None else valid_count.data_ptr(),
-                       kernel, tune, layout, F32)
-    # planar tensors and ragged channel counts: lend the scratch of the largest level (the levels run one after another)
-    need = 0
-    for f, hw in zip(features, hws):
-        base.features, base.feat_h, base.feat_w = f.data_ptr(), hw[0], hw[1]
-        need = max(need, flashbev_workspace_bytes(base))
-    base.features, base.feat_h, base.feat_w = f0.data_ptr(), hws[0][0], hws[0][1]
-    if need:
-        ws = torch.empty(need, dtype=torch.uint8, device=f0.device)
-        base.workspace, base.workspace_bytes = ws.data_ptr(), need
-    if stream is None:
-        stream = torch.cuda.current_stream(f0.device).cuda_stream
-    with torch.cuda.device(f0.device):
-        flashbev_sampling_vt_multires(base, [f.data_ptr() for f in features], hws, stream)
-    return out
+    return _result((_native or native()).sampling_vt_multires(features, lidar2img, img_hw, bev_range, grid, reduce, out,
+                                                              valid_count, kernel, tune, stream, layout),
+                   "flashbev_sampling_vt_multires")

@@ -1,8 +1,10 @@
-"""Build the CUDA library in-tree for sm_100a (nvcc cross-compiles without a GPU)."""
+"""Build the CUDA library in-tree for sm_100a (nvcc cross-compiles without a GPU) and its CPython entry points."""
 from __future__ import annotations
 
+import importlib.util
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(_HERE)
@@ -17,6 +19,10 @@ NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a",
 LIB_DEBUG_BOUNDS = os.path.join(_HERE, "libflashbev_debug_bounds.so")
 
 
+NATIVE_SOURCES = [os.path.join(_HERE, "csrc", "native.cpp")]
+NATIVE = os.path.join(_HERE, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
+
+
 def needs_build(lib: str = LIB) -> bool:
     if not os.path.exists(lib):
         return True
@@ -24,8 +30,23 @@ def needs_build(lib: str = LIB) -> bool:
     return any(os.path.getmtime(s) > t for s in SOURCES + HEADERS)
 
 
+def build_native(force: bool = False) -> str:
+    """Compile csrc/native.cpp (g++, PyTorch headers) into the extension module next to this file; returns its path."""
+    sources = NATIVE_SOURCES + HEADERS[:1]
+    if force or not os.path.exists(NATIVE) or any(os.path.getmtime(s) > os.path.getmtime(NATIVE) for s in sources):
+        torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
+        inc = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
+               sysconfig.get_paths()["include"], "/usr/local/cuda/include", os.path.join(ROOT, "include")]
+        cmd = ([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-w"] +
+               [f"-I{d}" for d in inc] + NATIVE_SOURCES +
+               [f"-L{os.path.join(torch_dir, 'lib')}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
+                f"-L{_HERE}", "-lflashbev", "-Wl,-rpath,$ORIGIN", "-o", NATIVE])
+        subprocess.run(cmd, check=True)
+    return NATIVE
+
+
 def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False) -> str:
-    """Compile csrc/*.cu into libflashbev.so next to this file; returns its path.
+    """Compile csrc/*.cu into libflashbev.so next to this file (and the extension module over it); returns its path.
 
     ``debug_bounds``: build libflashbev_debug_bounds.so instead, with -DFLASHBEV_DEBUG_BOUNDS: every index the
     tiled kernel computes is range-checked, violations are counted into the caller's ``debug_error_word`` and
@@ -36,6 +57,8 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
         cmd = ([nvcc] + NVCC_FLAGS + (["-DFLASHBEV_DEBUG_BOUNDS"] if debug_bounds else []) +
                (["-Xptxas", "-v"] if verbose else []) + SOURCES + ["-o", lib])
         subprocess.run(cmd, check=True)
+    if not debug_bounds:
+        build_native(force)
     return lib
 
 
