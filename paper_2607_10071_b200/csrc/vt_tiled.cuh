@@ -314,8 +314,8 @@ __device__ __forceinline__ int column_build(const KParams &p, const double *mats
         while (khi > klo && !inside(khi)) --khi;
         if (klo > khi) return 0;
         const bool rev = sy < 0.0;  // rows ascend with the renumbered bins k' = khi - k
-        const double flx = floor(fx);
-        const int x0 = (int)flx;
+        double flx;
+        const int x0 = floor_int(fx, flx);
         const int edge = x0 < 0 ? 1 : (x0 >= p.Wf - 1 ? 2 : 0);
         const int xc = edge == 1 ? 0 : (edge == 2 ? max(p.Wf - 2, 0) : x0);
         D.d0 = fma((double)(rev ? khi : klo), sy, ay);
@@ -380,7 +380,8 @@ __device__ __forceinline__ bool affine_by_rows(const ColDesc &D) { return D.d1 <
 // Units (rows or bins) of an affine column that its runs are cut from, and the first row it writes.
 __device__ __forceinline__ int affine_units(const KParams &p, const ColDesc &D, int nb, int &row_first)
 {
-    const int r_first = (int)floor(D.d0), r_last = (int)floor(fma((double)(nb - 1), D.d1, D.d0));
+    double fl;
+    const int r_first = floor_int(D.d0, fl), r_last = floor_int(fma((double)(nb - 1), D.d1, D.d0), fl);
     row_first = max(r_first, 0);
     return affine_by_rows(D) ? max(0, min(r_last + 1, p.Hf - 1) - row_first + 1) : nb;
 }
@@ -437,8 +438,9 @@ __device__ __forceinline__ void walk_affine(const KParams &p, const WarpSmem &sm
         double kd = (double)kb;
         const unsigned char *dk = den + kb * dstep;
         for (int k = kb; k < ke; ++k, kd += 1.0, dk += dstep) {
-            const double fy = fma(kd, S, A), fl = floor(fy);
-            const int i = (int)fl - ra;  // row of the upper tap, relative: -1 .. len - 1, never decreasing
+            const double fy = fma(kd, S, A);
+            double fl;
+            const int i = floor_int(fy, fl) - ra;  // row of the upper tap, relative: -1 .. len - 1, never decreasing
             float ty = (float)(fy - fl), tu = 1.f - ty;
             if (eq1) {
 #ifdef FLASHBEV_DEBUG_BOUNDS
@@ -470,8 +472,9 @@ __device__ __forceinline__ void walk_affine(const KParams &p, const WarpSmem &sm
         double kd = (double)u0;
         const unsigned char *dk = den + u0 * dstep;
         for (int i = 0; i < len; ++i, kd += 1.0, dk += dstep) {
-            const double fy = fma(kd, S, A), fl = floor(fy);
-            const int r = (int)fl;
+            const double fy = fma(kd, S, A);
+            double fl;
+            const int r = floor_int(fy, fl);
             float ty = (float)(fy - fl), tu = 1.f - ty;
             if (eq1) {
 #ifdef FLASHBEV_DEBUG_BOUNDS
@@ -527,8 +530,8 @@ __device__ __forceinline__ int walk_general(const KParams &p, const WarpSmem &sm
             const double rd = fast_rcp(d);
             const double fx = fma(fma(m[2], zw, D.d0), rd, -0.5);
             const double fy = fma(fma(m[6], zw, D.d1), rd, -0.5);
-            const double flx = floor(fx), fly = floor(fy);
-            r[i] = (int)fly, x0[i] = (int)flx;
+            double flx, fly;
+            r[i] = floor_int(fy, fly), x0[i] = floor_int(fx, flx);
             ty[i] = (float)(fy - fly);
             fold_x(x0[i], (float)(fx - flx), p.Wf, xc[i], cl[i], cr[i]);
         }
