@@ -67,6 +67,7 @@ struct KParams {
     int whole_tasks;            // super-blocks (in visiting order) taken whole by one warp; the rest go one sub-block per warp
     int walk, walk_shift;       // height bins (or texel rows) per run: a power of two, 2 walk <= slots
     int inv_g;                  // ceil(65536 / g)
+    int inv_cpw;                // ceil(65536 / cpw)
     int slots;                  // record slots per warp
     int colcap;                 // column descriptors per warp (>= cpw * N)
     int wcap;                   // runs per warp (= column descriptors per warp * ceil(Z / walk))
@@ -973,6 +974,7 @@ flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V,
     if (cpw == 5 || cpw == 7) k.wy = cpw;
     k.wx = cpw / k.wy;
     k.cpw = k.wx * k.wy;
+    k.inv_cpw = (65536 + k.cpw - 1) / k.cpw;
 
     // record slots per warp and bins per run (a run writes at most two records per bin)
     const int slots_tune = (p->tune[3] >> 20) & 0xff;

@@ -814,6 +814,7 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
         const int ix0 = bx * (p.sbx * p.wx), iy0 = by * (p.sby * p.wy);
 
         unsigned in_mask;  // bit c: cell c of the super-block is inside the grid
+        int my_ocell;      // output row of cell `lane`
         {
             const int lx = my_tab & 0xff, ly = my_tab >> 8;
             const bool in = (lane >= s_begin * p.cpw) && (lane < s_end * p.cpw) && (ix0 + lx < p.X) && (iy0 + ly < p.Y);
@@ -822,6 +823,7 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                 sm.cellxy[lane] = make_double2(in ? p.x_min + ((double)(ix0 + lx) + 0.5) * p.dx : nan,
                                                in ? p.y_min + ((double)(iy0 + ly) + 0.5) * p.dy : nan);
             in_mask = __ballot_sync(FULL, in);
+            my_ocell = in ? (int)FB_IDX(((size_t)b * p.X + (ix0 + lx)) * p.Y + (iy0 + ly), (size_t)p.B * p.X * p.Y, p.err) : 0;  // < 2^31
         }
         __syncwarp();
         survey_candidates(p, cx, in_mask);
@@ -834,31 +836,35 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
             const int ncols = sm.cfirst[min(s1 * p.cpw, p.ct)] - jb;  // <= colcap: a sub-block has at most cpw * N candidates
             const int nw = build_columns(p, cx, jb, ncols, s0 * p.cpw, min(s1 * p.cpw, p.ct));
 
+            // ---- the records [r0, r1) of the cell this lane stands for (lane = cell of the super-block), counted from the
+            // segment's first: the sub-block loop below gets what it needs of them by shuffles (through the tables in shared
+            // memory every sub-block paid three dependent look-ups for each of its bounds)
+            int r0 = 0, r1 = 0;
+            if (lane >= s0 * p.cpw && lane < min(s1 * p.cpw, p.ct))
+                r0 = sm.woff[sm.colw[sm.cfirst[lane] - jb]], r1 = sm.woff[sm.colw[sm.cfirst[lane + 1] - jb]];
+
             // ---- rounds: the runs of as many whole sub-blocks as fit the record slots are walked together (one lane
             // per run), then the sub-blocks are gathered one by one
-            int wa = 0, wb = 0;  // the current round holds runs [wa, wb)
+            int round_end = s0, base = 0;  // the current round holds the records of sub-blocks before round_end, from `base` on
             for (int s = s0; s < s1; ++s) {
-                const int cell = s * p.cpw + (role ? cg : 0);
+                const int first = s * p.cpw, cell = first + (role ? cg : 0);
                 const bool lane_on = role && ((in_mask >> cell) & 1u);
-                const int tab = celltab[cell];
                 // (lanes without a cell inside the grid never use it)
-                const size_t ocell = lane_on ? (size_t)FB_IDX(((size_t)b * p.X + (ix0 + (tab & 0xff))) * p.Y + (iy0 + (tab >> 8)),
-                                                              (size_t)p.B * p.X * p.Y, p.err) : 0;
-                const int sw_lo = sm.colw[sm.cfirst[s * p.cpw] - jb], sw_hi = sm.colw[sm.cfirst[min((s + 1) * p.cpw, p.ct)] - jb];
-                const int cw_lo = sm.colw[sm.cfirst[cell] - jb], cw_hi = sm.colw[sm.cfirst[cell + 1] - jb];  // this lane's cell
-                const int sub_records = sm.woff[sw_hi] - sm.woff[sw_lo];
-                const bool oversized = sub_records > p.slots;
-                if (!oversized && sw_hi > wb) {
-                    __syncwarp();
-                    wa = sw_lo, wb = sw_hi;
-                    for (int s2 = s + 1; s2 < s1; ++s2) {
-                        const int hi2 = sm.colw[sm.cfirst[min((s2 + 1) * p.cpw, p.ct)] - jb];
-                        if (sm.woff[hi2] - sm.woff[wa] > p.slots) break;
-                        wb = hi2;
+                const size_t ocell = (size_t)(unsigned)__shfl_sync(FULL, my_ocell, cell);
+                const int cr0 = __shfl_sync(FULL, r0, cell), cr1 = __shfl_sync(FULL, r1, cell);  // this lane's cell
+                bool oversized = false;
+                if (s >= round_end) {
+                    base = __shfl_sync(FULL, r0, first);
+                    // cells from `first` on whose records all fit: a prefix, cut to whole sub-blocks
+                    const unsigned fits = __ballot_sync(FULL, lane >= first && lane < min(s1 * p.cpw, p.ct) && r1 - base <= p.slots);
+                    round_end = s + (__popc(fits) * p.inv_cpw >> 16);
+                    oversized = round_end == s;
+                    if (!oversized) {
+                        __syncwarp();
+                        const int wa = sm.colw[sm.cfirst[first] - jb], wb = sm.colw[sm.cfirst[round_end * p.cpw] - jb];
+                        for (int w = wa + lane; w < wb; w += 32) walk_one(p, sm, mats, w, sm.woff[w] - base);
+                        __syncwarp();
                     }
-                    const int base = sm.woff[wa];
-                    for (int w = wa + lane; w < wb; w += 32) walk_one(p, sm, mats, w, sm.woff[w] - base);
-                    __syncwarp();
                 }
 
                 float2 acc[V][PV];
@@ -876,7 +882,7 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                         const int vi = vec0 + v * vstep;
                         go[v] = make_float4(0.f, 0.f, 0.f, 0.f);
                         on[v] = lane_on && vi < p.vecs;
-                        if (on[v] && cw_hi > cw_lo) {
+                        if (on[v] && cr1 > cr0) {
                             go[v] = __ldg(reinterpret_cast<const float4 *>(p.gout + ocell * p.C) + vi);
                             go[v].x *= gscale, go[v].y *= gscale, go[v].z *= gscale, go[v].w *= gscale;
                         }
@@ -884,8 +890,8 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                 }
 
                 if (!oversized) {
-                    const int c0 = sm.woff[cw_lo] - sm.woff[wa];
-                    const int nrec = lane_on ? sm.woff[cw_hi] - sm.woff[cw_lo] : 0;
+                    const int c0 = cr0 - base;
+                    const int nrec = lane_on ? cr1 - cr0 : 0;
                     if (BWD) {
                         if (nrec > 0) scatter_list<V>(go, on, sm.roff + c0, sm.rw + c0, nrec, p.rstep, gfv);
                     } else {
@@ -894,10 +900,12 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                 } else {
                     // A sub-block whose records exceed the slots: several rounds of as many runs as fit, in order; the
                     // accumulators live across the walkers here.
+                    const int sw_lo = sm.colw[sm.cfirst[first] - jb], sw_hi = sm.colw[sm.cfirst[first + p.cpw] - jb];
+                    const int cw_lo = sm.colw[sm.cfirst[cell] - jb], cw_hi = sm.colw[sm.cfirst[cell + 1] - jb];
                     int pos = sw_lo;
                     while (pos < sw_hi) {
                         __syncwarp();
-                        const int base = sm.woff[pos];
+                        base = sm.woff[pos];
                         int upto = pos;
                         for (int w0 = pos + 1; w0 <= sw_hi; w0 += 32) {
                             const int w = w0 + lane;
@@ -920,7 +928,7 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                         }
                         pos = upto;
                     }
-                    wa = wb = sw_hi;
+                    round_end = s + 1;
                 }
                 if (BWD) continue;
 
