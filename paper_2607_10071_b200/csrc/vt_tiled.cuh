@@ -57,7 +57,6 @@
 constexpr int kMaxCt = 32;   // cells per super-block
 constexpr int kMaxCpw = 8;   // cells per sub-block
 constexpr int kColCapMax = 64;  // column descriptors per warp (a sub-block never has more candidates than that)
-constexpr int kWalkIlp = 1;  // height bins whose geometry a general walker evaluates independently
 
 struct __align__(16) ColDesc {
     double d0, d1;  // affine: fy(k') = d0 + k' d1 with d1 >= 0 (bins renumbered so that rows ascend); general: a0, a1
@@ -494,79 +493,118 @@ __device__ __forceinline__ void walk_affine(const KParams &p, const WarpSmem &sm
     }
 }
 
-// ---- step 2: walker of a general column (every bin projected in fp64).  COUNT-only or EMIT. ------------------------
-template <bool EMIT>
-__device__ __forceinline__ int walk_general(const KParams &p, const WarpSmem &sm, const double *mats, const ColDesc &D, int k0,
-                                            int len, int *out_off, float2 *out_w, int cap)
+// ---- step 2 of a segment with general columns: a lane per sample, 32 samples at a time -------------------------------
+// The samples of the segment's columns are numbered through (column by column, bins so that rows ascend); samples [from, to)
+// are projected in fp64, each exactly once and independently of the others, and become records on the fly: a sample in the
+// same texel rows as the one before it adds to that one's two records, one a row further down shares a record with it, any
+// other starts two.  Two ballots number the records; the weights of a chain of samples in the same rows are pulled together
+// by its first lane.  (One lane per column, bin after bin, and once more to count the records first, was a third of all
+// instructions on calibrated rigs: most lanes idle, every bin a chain of dependent fp64 operations.)
+// q0, q1: sample numbers of this lane's choice; r0, r1: how many records precede them.
+__device__ __forceinline__ void emit_samples(const KParams &p, const WarpSmem &sm, const double *mats, int nonempty, int from, int to, int q0,
+                                             int q1, int &r0, int &r1)
 {
-    const int meta = D.meta;
-    const bool rev = (meta >> 13) & 1;
-    const int cell = meta & 63, cam = (meta >> 6) & 63;
-    const int klo = D.kk & 0xffff, khi = (D.kk >> 16) & 0xffff;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt_mask = (1u << lane) - 1u, le_mask = lt_mask | (1u << lane);
     const int rowv = p.Wf * p.vecs;
-    const double *m = mats + cam * 12;
     const double zc0 = p.z_min + 0.5 * p.dz;
-    int n = 0;
-    bool open = false;
-    int ro = 0, xo = 0, xco = 0;  // open rows (ro, ro + 1) at bilinear corner column xo, first loaded texel xco
-    float uL = 0.f, uR = 0.f, lL = 0.f, lR = 0.f;
-    auto put = [&](int row, float wl, float wr) {
-        if (row >= 0 && row <= p.Hf - 1) {
-            if (EMIT && n < cap) {
-                const int off = FB_IDX((cam * p.Hf * p.Wf + xco) * p.vecs + row * rowv, p.nvec_cam - p.vecs - p.rstep + 1, p.err);
-                out_off[n] = off, out_w[n] = make_float2(wl, wr);
+    const int st0 = lane < nonempty ? sm.woff[lane] : 0x7fffffff, st1 = lane + 32 < nonempty ? sm.woff[lane + 32] : 0x7fffffff;
+    int base = 0;
+    r0 = r1 = 0;
+    for (int ps = from; ps < to; ps += 32) {
+        // columns that start in this window of samples, and those before it
+        unsigned starts = 0u;
+        if ((unsigned)(st0 - ps) < 32u) starts = 1u << (st0 - ps);
+        if ((unsigned)(st1 - ps) < 32u) starts |= 1u << (st1 - ps);
+        starts = __reduce_or_sync(FULL, starts);
+        const int before = __popc(__ballot_sync(FULL, st0 < ps)) + __popc(__ballot_sync(FULL, st1 < ps));
+        const bool on = ps + lane < to;
+        int x0 = 0, r = 0, off = 0;
+        float2 u = make_float2(0.f, 0.f), l = u;  // weights of the left and right texel in the sample's upper and lower row
+        if (on) {
+            const int m = before + __popc(starts & le_mask) - 1;
+            const ColDesc D = sm.col[FB_IDX(sm.wk[FB_IDX(m, p.wcap, p.err)], p.colcap, p.err)];
+            const int kp = ps + lane - sm.woff[m];
+            const int klo = D.kk & 0xffff, khi = (D.kk >> 16) & 0xffff, meta = D.meta;
+            const int k = (meta >> 13) & 1 ? khi - kp : klo + kp;
+            float cl, cr, ty;
+            double fl;
+            if ((meta >> 12) & 1) {  // affine
+                const double fy = fma((double)kp, D.d1, D.d0);
+                r = floor_int(fy, fl);
+                ty = (float)(fy - fl);
+                const int edge = (meta >> 14) & 3;
+                const float tx = D.f.tx;
+                cl = edge == 0 ? 1.f - tx : (edge == 1 ? tx : (p.Wf > 1 ? 0.f : 1.f - tx));
+                cr = edge == 0 ? tx : (edge == 2 && p.Wf > 1 ? 1.f - tx : 0.f);
+                off = D.f.offc;
+            } else {
+                const int cam = (meta >> 6) & 63;
+                const double *M = mats + cam * 12;
+                const double zw = fma((double)k, p.dz, zc0);
+                const double rd = fast_rcp(fma(M[10], zw, D.d2));
+                const double fx = fma(fma(M[2], zw, D.d0), rd, -0.5), fy = fma(fma(M[6], zw, D.d1), rd, -0.5);
+                x0 = floor_int(fx, fl);
+                const float tx = (float)(fx - fl);
+                r = floor_int(fy, fl);
+                ty = (float)(fy - fl);
+                int xc;
+                fold_x(x0, tx, p.Wf, xc, cl, cr);
+                off = (cam * p.Hf * p.Wf + xc) * p.vecs;
             }
-            ++n;
+            float tu = 1.f - ty;
+            if (p.reduce == FLASHBEV_REDUCE_CAMERA_MEAN_Z_SUM) {  // Eq. 1: 1 / max(1, cameras that see this height)
+                const unsigned dn = sm.den[FB_IDX((meta & 63) * p.Z + k, p.den_bytes, p.err)];
+                const float sc = 1.f / (float)(dn > 1u ? dn : 1u);
+                ty *= sc, tu *= sc;
+            }
+            u = make_float2(cl * tu, cr * tu), l = make_float2(cl * ty, cr * ty);
         }
-    };
-    for (int i0 = 0; i0 < len; i0 += kWalkIlp) {
-        int r[kWalkIlp], x0[kWalkIlp], xc[kWalkIlp];
-        float cl[kWalkIlp], cr[kWalkIlp], ty[kWalkIlp];
-#pragma unroll
-        for (int i = 0; i < kWalkIlp; ++i) {
-            const int kp = k0 + min(i0 + i, len - 1);  // past the end: the last bin again (ignored below)
-            const double zw = fma((double)(rev ? khi - kp : klo + kp), p.dz, zc0);
-            const double d = fma(m[10], zw, D.d2);
-            const double rd = fast_rcp(d);
-            const double fx = fma(fma(m[2], zw, D.d0), rd, -0.5);
-            const double fy = fma(fma(m[6], zw, D.d1), rd, -0.5);
-            double flx, fly;
-            r[i] = floor_int(fy, fly), x0[i] = floor_int(fx, flx);
-            ty[i] = (float)(fy - fly);
-            fold_x(x0[i], (float)(fx - flx), p.Wf, xc[i], cl[i], cr[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < kWalkIlp; ++i) {
-            if (i0 + i < len) {
-                const bool col_same = open & (x0[i] == xo);
-                const bool same = col_same & (r[i] == ro), next = col_same & (r[i] == ro + 1);
-                if (!same) {
-                    if (open) {
-                        put(ro, uL, uR);
-                        if (!next) put(ro + 1, lL, lR);
-                    }
-                    uL = next ? lL : 0.f, uR = next ? lR : 0.f, lL = 0.f, lR = 0.f;
-                    ro = r[i], xo = x0[i], xco = xc[i], open = true;
-                }
-                if (EMIT) {
-                    float s = 1.f;
-                    if (p.reduce == FLASHBEV_REDUCE_CAMERA_MEAN_Z_SUM) {  // Eq. 1: 1 / max(1, cameras that see this height)
-                        const int kp = k0 + i0 + i;
-                        const unsigned dn = sm.den[FB_IDX(cell * p.Z + (rev ? khi - kp : klo + kp), p.den_bytes, p.err)];
-                        s = 1.f / (float)(dn > 1u ? dn : 1u);
-                    }
-                    const float wy1 = ty[i] * s, wy0 = (1.f - ty[i]) * s;
-                    uL = fmaf(cl[i], wy0, uL), uR = fmaf(cr[i], wy0, uR);
-                    lL = fmaf(cl[i], wy1, lL), lR = fmaf(cr[i], wy1, lR);
-                }
+        const int px = __shfl_up_sync(FULL, x0, 1), pr = __shfl_up_sync(FULL, r, 1);
+        const bool link = on && lane > 0 && !((starts >> lane) & 1u) && px == x0;  // same column as the lane before, same texel columns
+        const bool same = link && pr == r, next = link && pr + 1 == r;
+        const unsigned sames = __ballot_sync(FULL, same), nexts = __ballot_sync(FULL, next);
+        int len = 0;  // samples after this one that are in the same rows
+        if (sames) {
+            len = lane < 31 ? __ffs(~(sames >> (lane + 1))) - 1 : 0;
+            if (same) len = 0;
+            for (int d = 1; __any_sync(FULL, d <= len); ++d) {
+                const float a = __shfl_down_sync(FULL, u.x, d), b = __shfl_down_sync(FULL, u.y, d);
+                const float c = __shfl_down_sync(FULL, l.x, d), e = __shfl_down_sync(FULL, l.y, d);
+                // (lanes inside a chain keep their own weights: only heads have len > 0)
+                if (d <= len) u.x += a, u.y += b, l.x += c, l.y += e;
             }
         }
+        if (nexts) {  // the lower row of a chain is the upper row of the one after it
+            const int e = lane + len + 1;
+            const float a = __shfl_sync(FULL, u.x, e & 31), b = __shfl_sync(FULL, u.y, e & 31);
+            if (!same && e < 32 && ((nexts >> e) & 1u)) l.x += a, l.y += b;
+        }
+        const bool up = on && !same && !next && r >= 0, dn = on && !same && r + 1 <= p.Hf - 1;
+        const unsigned ups = __ballot_sync(FULL, up), dns = __ballot_sync(FULL, dn);
+        int at = base + __popc(ups & lt_mask) + __popc(dns & lt_mask);
+        if (up) {
+            at = FB_IDX(at, p.slots, p.err);
+            sm.roff[at] = FB_IDX(off + r * rowv, p.nvec_cam - p.vecs - p.rstep + 1, p.err), sm.rw[at] = u;
+            ++at;
+        }
+        if (dn) {
+            at = FB_IDX(at, p.slots, p.err);
+            sm.roff[at] = FB_IDX(off + (r + 1) * rowv, p.nvec_cam - p.vecs - p.rstep + 1, p.err), sm.rw[at] = l;
+        }
+        if ((unsigned)(q0 - ps) < 32u) {
+            const unsigned b = (1u << (q0 - ps)) - 1u;
+            r0 = base + __popc(ups & b) + __popc(dns & b);
+        }
+        if ((unsigned)(q1 - ps) < 32u) {
+            const unsigned b = (1u << (q1 - ps)) - 1u;
+            r1 = base + __popc(ups & b) + __popc(dns & b);
+        }
+        base += __popc(ups) + __popc(dns);
     }
-    if (open) {
-        put(ro, uL, uR);
-        put(ro + 1, lL, lR);
-    }
-    return n;
+    if (q0 >= to) r0 = base;
+    if (q1 >= to) r1 = base;
 }
 
 // The three geometry steps are separate functions (not inlined) so that their fp64-heavy register needs stay out of
@@ -610,29 +648,54 @@ __device__ __forceinline__ int survey_candidates(const KParams &p, WarpCtx cx, u
     return nsurv;
 }
 
-// ---- step 1b over a segment (survivors [jb, jb + ncols), cells [c_lo, c_hi)): exact intervals, runs and their record
-// counts (two exclusive scans over the columns), valid samples per cell, Eq. 1 camera counts.  Returns the number of runs.
+// ---- step 1b over a segment (survivors [jb, jb + ncols), cells [c_lo, c_hi)): exact intervals, valid samples per cell,
+// Eq. 1 camera counts.  A segment of affine columns only: runs and their record counts (two exclusive scans over the columns);
+// returns 0.  With a general column among them: the columns that have bins, in order (wk), and where their samples start when
+// they are numbered through (woff; colw for every column); returns 1 + the number of those columns.
 __device__ __forceinline__ int build_columns(const KParams &p, WarpCtx cx, int jb, int ncols, int c_lo, int c_hi)
 {
     constexpr unsigned FULL = 0xffffffffu;
     const WarpSmem sm = warp_smem(p, cx.warp_base);
     const int lane = threadIdx.x & 31;
+    bool general = false;
+    for (int j = lane; j < ncols; j += 32) {
+        ColDesc D;
+        const int cn = sm.cand[jb + j];
+        const int nb = column_build(p, cx.mats, cx.slope, cx.camfast, sm.cellxy[cn & 0xff], cn & 0xff, cn >> 8, D);
+        sm.col[FB_IDX(j, p.colcap, p.err)] = D;
+        general |= nb > 0 && !((D.meta >> 12) & 1);
+    }
+    general = __any_sync(FULL, general);
     int nw = 0, nrec_seg = 0;
     for (int j0 = 0; j0 < ncols; j0 += 32) {
         const int j = j0 + lane;
         ColDesc D;
         int nb = 0;
         if (j < ncols) {
-            const int cn = sm.cand[jb + j];
-            nb = column_build(p, cx.mats, cx.slope, cx.camfast, sm.cellxy[cn & 0xff], cn & 0xff, cn >> 8, D);
-            sm.col[FB_IDX(j, p.colcap, p.err)] = D;
+            D = sm.col[j];  // (this lane's own)
+            nb = ((D.kk >> 16) & 0xffff) - (D.kk & 0xffff) + 1;
         }
-        bool affine = false;
-        int units = nb, row_first = 0;  // what the column's runs are cut from: bins, or rows of an affine column
-        if (nb > 0) {
-            affine = (D.meta >> 12) & 1;
-            if (affine) units = affine_units(p, D, nb, row_first);
+        if (general) {
+            const unsigned some = __ballot_sync(FULL, nb > 0);
+            int x = nb;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(FULL, x, off);
+                if (lane >= off) x += y;
+            }
+            const int start = nrec_seg + x - nb;
+            if (j < ncols) {
+                sm.colw[j] = start;
+                if (nb > 0) {
+                    const int m = nw + __popc(some & ((1u << lane) - 1u));
+                    sm.wk[FB_IDX(m, p.wcap, p.err)] = (uint32_t)j, sm.woff[FB_IDX(m, p.wcap + 1, p.err)] = start;
+                }
+            }
+            nrec_seg += __shfl_sync(FULL, x, 31), nw += __popc(some);
+            continue;
         }
+        int units = nb, row_first = 0;  // what the column's runs are cut from: rows, or bins of a column with steps of several rows
+        if (nb > 0) units = affine_units(p, D, nb, row_first);
         const int runs = (units + p.walk - 1) >> p.walk_shift;  // walk is a power of two
         int x = runs;
 #pragma unroll
@@ -651,7 +714,7 @@ __device__ __forceinline__ int build_columns(const KParams &p, WarpCtx cx, int j
                 const int u0 = i * per, len = min(per, units - u0);
                 sm.wk[FB_IDX(wbase + i, p.wcap, p.err)] = (uint32_t)j | ((uint32_t)u0 << 8) | ((uint32_t)(len - 1) << 24);
                 sm.woff[FB_IDX(wbase + i, p.wcap + 1, p.err)] = mine;
-                mine += affine ? affine_run_records(D, len) : walk_general<false>(p, sm, cx.mats, D, u0, len, nullptr, nullptr, 0);
+                mine += affine_run_records(D, len);
             }
         }
         int y = mine;
@@ -665,7 +728,10 @@ __device__ __forceinline__ int build_columns(const KParams &p, WarpCtx cx, int j
         if (j < ncols)
             for (int i = 0; i < runs; ++i) sm.woff[wbase + i] += rbase;
     }
-    if (lane == 0) sm.colw[ncols] = nw, sm.woff[nw] = nrec_seg;
+    if (lane == 0) {
+        sm.colw[ncols] = general ? nrec_seg : nw;
+        if (!general) sm.woff[nw] = nrec_seg;
+    }
     __syncwarp();
 
     // valid samples per cell; Eq. 1: cameras per (cell, height bin) -- the intervals say it all
@@ -689,17 +755,16 @@ __device__ __forceinline__ int build_columns(const KParams &p, WarpCtx cx, int j
         }
     }
     __syncwarp();
-    return nw;
+    return general ? nw + 1 : 0;
 }
 
-// ---- step 2: run w is walked by the calling lane; its records go to slots [at, at + its count) ------------------
-__device__ __forceinline__ void walk_one(const KParams &p, const WarpSmem &sm, const double *mats, int w, int at)
+// ---- step 2: run w of an affine column is walked by the calling lane; its records go to slots [at, at + its count) ----
+__device__ __forceinline__ void walk_one(const KParams &p, const WarpSmem &sm, int w, int at)
 {
     const uint32_t wd = sm.wk[w];
     const ColDesc D = sm.col[FB_IDX(wd & 0xff, p.colcap, p.err)];
     at = FB_IDX(at, p.slots, p.err);
-    if ((D.meta >> 12) & 1) walk_affine(p, sm, D, (wd >> 8) & 0xffff, (wd >> 24) + 1, sm.roff + at, sm.rw + at, p.slots - at);
-    else walk_general<true>(p, sm, mats, D, (wd >> 8) & 0xffff, (wd >> 24) + 1, sm.roff + at, sm.rw + at, p.slots - at);
+    walk_affine(p, sm, D, (wd >> 8) & 0xffff, (wd >> 24) + 1, sm.roff + at, sm.rw + at, p.slots - at);
 }
 
 // WIDE: a lane's V channel vectors are adjacent (32-byte aligned pairs, 256-bit loads) instead of g apart
@@ -834,38 +899,52 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
             int s1 = s0 + 1;
             while (s1 < s_end && sm.cfirst[min((s1 + 1) * p.cpw, p.ct)] - jb <= p.colcap) ++s1;
             const int ncols = sm.cfirst[min(s1 * p.cpw, p.ct)] - jb;  // <= colcap: a sub-block has at most cpw * N candidates
-            const int nw = build_columns(p, cx, jb, ncols, s0 * p.cpw, min(s1 * p.cpw, p.ct));
+            const int general = build_columns(p, cx, jb, ncols, s0 * p.cpw, min(s1 * p.cpw, p.ct));  // 0, or 1 + columns that have bins
 
             // ---- the records [r0, r1) of the cell this lane stands for (lane = cell of the super-block), counted from the
             // segment's first: the sub-block loop below gets what it needs of them by shuffles (through the tables in shared
             // memory every sub-block paid three dependent look-ups for each of its bounds)
+            const int c_end = min(s1 * p.cpw, p.ct);
             int r0 = 0, r1 = 0;
-            if (lane >= s0 * p.cpw && lane < min(s1 * p.cpw, p.ct))
+            if (!general && lane >= s0 * p.cpw && lane < c_end)
                 r0 = sm.woff[sm.colw[sm.cfirst[lane] - jb]], r1 = sm.woff[sm.colw[sm.cfirst[lane + 1] - jb]];
 
             // ---- rounds: the runs of as many whole sub-blocks as fit the record slots are walked together (one lane
-            // per run), then the sub-blocks are gathered one by one
+            // per run; with general columns one lane per sample, two records each at most), then the sub-blocks are gathered
+            // one by one
             int round_end = s0, base = 0;  // the current round holds the records of sub-blocks before round_end, from `base` on
             for (int s = s0; s < s1; ++s) {
                 const int first = s * p.cpw, cell = first + (role ? cg : 0);
                 const bool lane_on = role && ((in_mask >> cell) & 1u);
                 // (lanes without a cell inside the grid never use it)
                 const size_t ocell = (size_t)(unsigned)__shfl_sync(FULL, my_ocell, cell);
-                const int cr0 = __shfl_sync(FULL, r0, cell), cr1 = __shfl_sync(FULL, r1, cell);  // this lane's cell
                 bool oversized = false;
-                if (s >= round_end) {
+                if (s >= round_end && general) {
+                    int q0 = 0, q1 = 0;  // samples of the cell this lane stands for
+                    if (lane >= first && lane < c_end) q0 = sm.colw[sm.cfirst[lane] - jb], q1 = sm.colw[sm.cfirst[lane + 1] - jb];
+                    const int from = __shfl_sync(FULL, q0, first);
+                    const unsigned fits = __ballot_sync(FULL, lane >= first && lane < c_end && 2 * (q1 - from) <= p.slots);
+                    round_end = s + (__popc(fits) * p.inv_cpw >> 16);
+                    oversized = round_end == s;
+                    if (!oversized) {
+                        __syncwarp();
+                        emit_samples(p, sm, mats, general - 1, from, __shfl_sync(FULL, q1, round_end * p.cpw - 1), q0, q1, r0, r1);
+                        __syncwarp();
+                    }
+                } else if (s >= round_end) {
                     base = __shfl_sync(FULL, r0, first);
                     // cells from `first` on whose records all fit: a prefix, cut to whole sub-blocks
-                    const unsigned fits = __ballot_sync(FULL, lane >= first && lane < min(s1 * p.cpw, p.ct) && r1 - base <= p.slots);
+                    const unsigned fits = __ballot_sync(FULL, lane >= first && lane < c_end && r1 - base <= p.slots);
                     round_end = s + (__popc(fits) * p.inv_cpw >> 16);
                     oversized = round_end == s;
                     if (!oversized) {
                         __syncwarp();
                         const int wa = sm.colw[sm.cfirst[first] - jb], wb = sm.colw[sm.cfirst[round_end * p.cpw] - jb];
-                        for (int w = wa + lane; w < wb; w += 32) walk_one(p, sm, mats, w, sm.woff[w] - base);
+                        for (int w = wa + lane; w < wb; w += 32) walk_one(p, sm, w, sm.woff[w] - base);
                         __syncwarp();
                     }
                 }
+                const int cr0 = __shfl_sync(FULL, r0, cell), cr1 = __shfl_sync(FULL, r1, cell);  // this lane's cell
 
                 float2 acc[V][PV];
 #pragma unroll
@@ -882,7 +961,7 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                         const int vi = vec0 + v * vstep;
                         go[v] = make_float4(0.f, 0.f, 0.f, 0.f);
                         on[v] = lane_on && vi < p.vecs;
-                        if (on[v] && cr1 > cr0) {
+                        if (on[v] && count > 0) {
                             go[v] = __ldg(reinterpret_cast<const float4 *>(p.gout + ocell * p.C) + vi);
                             go[v].x *= gscale, go[v].y *= gscale, go[v].z *= gscale, go[v].w *= gscale;
                         }
@@ -897,6 +976,26 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                     } else {
                         gather_list<V, BF16, kWide>(acc, roff_s + 4 * c0, rw_s + 8 * c0, nrec, (unsigned)p.rstep, featv);
                     }
+                } else if (general) {
+                    // A sub-block whose records may exceed the slots: several rounds of as many samples as are sure to fit
+                    int q0 = 0, q1 = 0;
+                    if (lane >= first && lane < first + p.cpw) q0 = sm.colw[sm.cfirst[lane] - jb], q1 = sm.colw[sm.cfirst[lane + 1] - jb];
+                    const int end = __shfl_sync(FULL, q1, first + p.cpw - 1);
+                    for (int from = __shfl_sync(FULL, q0, first); from < end;) {
+                        const int to = min(from + (p.slots >> 1), end);
+                        __syncwarp();
+                        emit_samples(p, sm, mats, general - 1, from, to, q0, q1, r0, r1);
+                        __syncwarp();
+                        const int c0 = __shfl_sync(FULL, r0, cell), c1 = __shfl_sync(FULL, r1, cell);
+                        const int nrec = lane_on ? c1 - c0 : 0;
+                        if (BWD) {
+                            if (nrec > 0) scatter_list<V>(go, on, sm.roff + c0, sm.rw + c0, nrec, p.rstep, gfv);
+                        } else {
+                            gather_list<V, BF16, kWide>(acc, roff_s + 4 * c0, rw_s + 8 * c0, nrec, (unsigned)p.rstep, featv);
+                        }
+                        from = to;
+                    }
+                    round_end = s + 1;
                 } else {
                     // A sub-block whose records exceed the slots: several rounds of as many runs as fit, in order; the
                     // accumulators live across the walkers here.
@@ -915,7 +1014,7 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                             if (bal != FULL) break;
                         }
                         if (upto <= pos) upto = pos + 1;  // (cannot happen: one run always fits; never loop without progress)
-                        for (int w = pos + lane; w < upto; w += 32) walk_one(p, sm, mats, w, sm.woff[w] - base);
+                        for (int w = pos + lane; w < upto; w += 32) walk_one(p, sm, w, sm.woff[w] - base);
                         __syncwarp();
                         // this lane's cell: its runs inside [pos, upto)
                         const int lw = min(max(cw_lo, pos), upto), hw = min(max(cw_hi, pos), upto);
