@@ -18,10 +18,10 @@
 //                   prefix sum over the record counts gives every run its place in the list, so the records of a
 //                   cell are contiguous, their order is fixed and no atomics are needed.  The valid-sample count
 //                   of a cell and the per-height camera counts of Eq. 1 follow from the intervals alone.
-//   2.  walkers     one lane per run: successive bins that land on the same texel rows are merged into one
-//                   record {left tap, right tap, wL, wR} per row.  Affine columns cost one fp64 FMA and a floor
-//                   per bin; the others are projected bin by bin in fp64 (their records are counted by a first
-//                   sweep of the same walker).
+//   2.  walkers     one lane per run of an affine column: successive bins that land on the same texel rows are merged
+//                   into one record {left tap, right tap, wL, wR} per row, at one fp64 FMA and a floor per bin.  Where a
+//                   segment holds a column of a tilted camera, one lane per sample instead: every sample is projected once
+//                   in fp64 and ballots number the records that the samples become.
 //   3.  gather      one sub-block at a time: g lanes per cell, V 16-byte channel vectors per lane; per record two
 //                   128- or 256-bit loads per vector and packed fp32 FMAs into register accumulators.  Runs that
 //                   do not fit the record slots are taken in several rounds; the accumulators of the sub-block
