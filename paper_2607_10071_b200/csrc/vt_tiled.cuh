@@ -500,8 +500,9 @@ __device__ __forceinline__ void walk_affine(const KParams &p, const WarpSmem &sm
 // other starts two.  Two ballots number the records; the weights of a chain of samples in the same rows are pulled together
 // by its first lane.  (One lane per column, bin after bin, and once more to count the records first, was a third of all
 // instructions on calibrated rigs: most lanes idle, every bin a chain of dependent fp64 operations.)
+// Stops where the record slots might not hold another 32 samples' records; returns the first sample not taken.
 // q0, q1: sample numbers of this lane's choice; r0, r1: how many records precede them.
-__device__ __forceinline__ void emit_samples(const KParams &p, const WarpSmem &sm, const double *mats, int nonempty, int from, int to, int q0,
+__device__ __forceinline__ int emit_samples(const KParams &p, const WarpSmem &sm, const double *mats, int nonempty, int from, int to, int q0,
                                              int q1, int &r0, int &r1)
 {
     constexpr unsigned FULL = 0xffffffffu;
@@ -512,7 +513,8 @@ __device__ __forceinline__ void emit_samples(const KParams &p, const WarpSmem &s
     const int st0 = lane < nonempty ? sm.woff[lane] : 0x7fffffff, st1 = lane + 32 < nonempty ? sm.woff[lane + 32] : 0x7fffffff;
     int base = 0;
     r0 = r1 = 0;
-    for (int ps = from; ps < to; ps += 32) {
+    int ps = from;
+    for (; ps < to && base + 64 <= p.slots; ps += 32) {
         // columns that start in this window of samples, and those before it
         unsigned starts = 0u;
         if ((unsigned)(st0 - ps) < 32u) starts = 1u << (st0 - ps);
@@ -603,8 +605,10 @@ __device__ __forceinline__ void emit_samples(const KParams &p, const WarpSmem &s
         }
         base += __popc(ups) + __popc(dns);
     }
+    to = min(ps, to);
     if (q0 >= to) r0 = base;
     if (q1 >= to) r1 = base;
+    return to;
 }
 
 // The three geometry steps are separate functions (not inlined) so that their fp64-heavy register needs stay out of
@@ -901,50 +905,22 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
             const int ncols = sm.cfirst[min(s1 * p.cpw, p.ct)] - jb;  // <= colcap: a sub-block has at most cpw * N candidates
             const int general = build_columns(p, cx, jb, ncols, s0 * p.cpw, min(s1 * p.cpw, p.ct));  // 0, or 1 + columns that have bins
 
-            // ---- the records [r0, r1) of the cell this lane stands for (lane = cell of the super-block), counted from the
-            // segment's first: the sub-block loop below gets what it needs of them by shuffles (through the tables in shared
-            // memory every sub-block paid three dependent look-ups for each of its bounds)
+            // ---- the units [q0, q1) of the cell this lane stands for (lane = cell of the super-block): runs, or samples if a
+            // column of the segment is general.  The sub-block loop gets what it needs of them by shuffles (through the tables in
+            // shared memory every sub-block paid three dependent look-ups for each of its bounds).
             const int c_end = min(s1 * p.cpw, p.ct);
-            int r0 = 0, r1 = 0;
-            if (!general && lane >= s0 * p.cpw && lane < c_end)
-                r0 = sm.woff[sm.colw[sm.cfirst[lane] - jb]], r1 = sm.woff[sm.colw[sm.cfirst[lane + 1] - jb]];
+            int q0 = 0, q1 = 0;
+            if (lane >= s0 * p.cpw && lane < c_end) q0 = sm.colw[sm.cfirst[lane] - jb], q1 = sm.colw[sm.cfirst[lane + 1] - jb];
 
-            // ---- rounds: the runs of as many whole sub-blocks as fit the record slots are walked together (one lane
-            // per run; with general columns one lane per sample, two records each at most), then the sub-blocks are gathered
-            // one by one
-            int round_end = s0, base = 0;  // the current round holds the records of sub-blocks before round_end, from `base` on
+            // ---- rounds: the records of as many whole sub-blocks as fit the slots are made together (one lane per run, or per
+            // sample), then the sub-blocks are gathered one by one
+            int round_end = s0;   // the current round holds the records of the sub-blocks before this one
+            int r0 = 0, r1 = 0;   // records of the cell this lane stands for
             for (int s = s0; s < s1; ++s) {
                 const int first = s * p.cpw, cell = first + (role ? cg : 0);
                 const bool lane_on = role && ((in_mask >> cell) & 1u);
                 // (lanes without a cell inside the grid never use it)
                 const size_t ocell = (size_t)(unsigned)__shfl_sync(FULL, my_ocell, cell);
-                bool oversized = false;
-                if (s >= round_end && general) {
-                    int q0 = 0, q1 = 0;  // samples of the cell this lane stands for
-                    if (lane >= first && lane < c_end) q0 = sm.colw[sm.cfirst[lane] - jb], q1 = sm.colw[sm.cfirst[lane + 1] - jb];
-                    const int from = __shfl_sync(FULL, q0, first);
-                    const unsigned fits = __ballot_sync(FULL, lane >= first && lane < c_end && 2 * (q1 - from) <= p.slots);
-                    round_end = s + (__popc(fits) * p.inv_cpw >> 16);
-                    oversized = round_end == s;
-                    if (!oversized) {
-                        __syncwarp();
-                        emit_samples(p, sm, mats, general - 1, from, __shfl_sync(FULL, q1, round_end * p.cpw - 1), q0, q1, r0, r1);
-                        __syncwarp();
-                    }
-                } else if (s >= round_end) {
-                    base = __shfl_sync(FULL, r0, first);
-                    // cells from `first` on whose records all fit: a prefix, cut to whole sub-blocks
-                    const unsigned fits = __ballot_sync(FULL, lane >= first && lane < c_end && r1 - base <= p.slots);
-                    round_end = s + (__popc(fits) * p.inv_cpw >> 16);
-                    oversized = round_end == s;
-                    if (!oversized) {
-                        __syncwarp();
-                        const int wa = sm.colw[sm.cfirst[first] - jb], wb = sm.colw[sm.cfirst[round_end * p.cpw] - jb];
-                        for (int w = wa + lane; w < wb; w += 32) walk_one(p, sm, w, sm.woff[w] - base);
-                        __syncwarp();
-                    }
-                }
-                const int cr0 = __shfl_sync(FULL, r0, cell), cr1 = __shfl_sync(FULL, r1, cell);  // this lane's cell
 
                 float2 acc[V][PV];
 #pragma unroll
@@ -968,67 +944,52 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                     }
                 }
 
-                if (!oversized) {
-                    const int c0 = cr0 - base;
-                    const int nrec = lane_on ? cr1 - cr0 : 0;
+                // A sub-block whose own records exceed the slots comes in several parts, in order; its accumulators stay in
+                // registers.  (One loop for both cases: every stage is in the kernel once, which small grids notice -- they run
+                // it through a cold instruction cache.)
+                int pos = __shfl_sync(FULL, q0, first);
+                const int end = __shfl_sync(FULL, q1, first + p.cpw - 1);
+                bool more;
+                do {
+                    if (s >= round_end) {
+                        const bool here = lane >= first && lane < c_end;
+                        __syncwarp();  // the records before have been taken
+                        unsigned fits;  // cells from `first` on whose records all fit: a prefix, cut to whole sub-blocks
+                        if (general) {
+                            const int to = emit_samples(p, sm, mats, general - 1, pos, __shfl_sync(FULL, q1, c_end - 1), q0, q1, r0, r1);
+                            fits = __ballot_sync(FULL, here && q1 <= to);
+                            pos = to;
+                        } else {
+                            const int base = sm.woff[pos];
+                            fits = __ballot_sync(FULL, here && sm.woff[q1] - base <= p.slots);
+                            const int whole = __popc(fits) * p.inv_cpw >> 16;
+                            int to = whole ? __shfl_sync(FULL, q1, (s + whole) * p.cpw - 1) : pos;
+                            if (whole == 0) {  // as many runs as fit
+                                for (int w0 = pos + 1; w0 <= end; w0 += 32) {
+                                    const int w = w0 + lane;
+                                    const unsigned bal = __ballot_sync(FULL, w <= end && sm.woff[w] - base <= p.slots);
+                                    to = w0 - 1 + __popc(bal);
+                                    if (bal != FULL) break;
+                                }
+                                to = max(to, pos + 1);  // (one run always fits; never loop without progress)
+                            }
+                            for (int w = pos + lane; w < to; w += 32) walk_one(p, sm, w, sm.woff[w] - base);
+                            r0 = sm.woff[min(max(q0, pos), to)] - base, r1 = sm.woff[min(max(q1, pos), to)] - base;
+                            pos = to;
+                        }
+                        __syncwarp();
+                        round_end = s + (__popc(fits) * p.inv_cpw >> 16);
+                        if (round_end == s && pos >= end) round_end = s + 1;
+                    }
+                    more = s >= round_end;
+                    const int c0 = __shfl_sync(FULL, r0, cell), c1 = __shfl_sync(FULL, r1, cell);  // this lane's cell
+                    const int nrec = lane_on ? c1 - c0 : 0;
                     if (BWD) {
                         if (nrec > 0) scatter_list<V>(go, on, sm.roff + c0, sm.rw + c0, nrec, p.rstep, gfv);
                     } else {
                         gather_list<V, BF16, kWide>(acc, roff_s + 4 * c0, rw_s + 8 * c0, nrec, (unsigned)p.rstep, featv);
                     }
-                } else if (general) {
-                    // A sub-block whose records may exceed the slots: several rounds of as many samples as are sure to fit
-                    int q0 = 0, q1 = 0;
-                    if (lane >= first && lane < first + p.cpw) q0 = sm.colw[sm.cfirst[lane] - jb], q1 = sm.colw[sm.cfirst[lane + 1] - jb];
-                    const int end = __shfl_sync(FULL, q1, first + p.cpw - 1);
-                    for (int from = __shfl_sync(FULL, q0, first); from < end;) {
-                        const int to = min(from + (p.slots >> 1), end);
-                        __syncwarp();
-                        emit_samples(p, sm, mats, general - 1, from, to, q0, q1, r0, r1);
-                        __syncwarp();
-                        const int c0 = __shfl_sync(FULL, r0, cell), c1 = __shfl_sync(FULL, r1, cell);
-                        const int nrec = lane_on ? c1 - c0 : 0;
-                        if (BWD) {
-                            if (nrec > 0) scatter_list<V>(go, on, sm.roff + c0, sm.rw + c0, nrec, p.rstep, gfv);
-                        } else {
-                            gather_list<V, BF16, kWide>(acc, roff_s + 4 * c0, rw_s + 8 * c0, nrec, (unsigned)p.rstep, featv);
-                        }
-                        from = to;
-                    }
-                    round_end = s + 1;
-                } else {
-                    // A sub-block whose records exceed the slots: several rounds of as many runs as fit, in order; the
-                    // accumulators live across the walkers here.
-                    const int sw_lo = sm.colw[sm.cfirst[first] - jb], sw_hi = sm.colw[sm.cfirst[first + p.cpw] - jb];
-                    const int cw_lo = sm.colw[sm.cfirst[cell] - jb], cw_hi = sm.colw[sm.cfirst[cell + 1] - jb];
-                    int pos = sw_lo;
-                    while (pos < sw_hi) {
-                        __syncwarp();
-                        base = sm.woff[pos];
-                        int upto = pos;
-                        for (int w0 = pos + 1; w0 <= sw_hi; w0 += 32) {
-                            const int w = w0 + lane;
-                            const bool fits = w <= sw_hi && sm.woff[w] - base <= p.slots;
-                            const unsigned bal = __ballot_sync(FULL, fits);
-                            upto = w0 - 1 + __popc(bal);
-                            if (bal != FULL) break;
-                        }
-                        if (upto <= pos) upto = pos + 1;  // (cannot happen: one run always fits; never loop without progress)
-                        for (int w = pos + lane; w < upto; w += 32) walk_one(p, sm, w, sm.woff[w] - base);
-                        __syncwarp();
-                        // this lane's cell: its runs inside [pos, upto)
-                        const int lw = min(max(cw_lo, pos), upto), hw = min(max(cw_hi, pos), upto);
-                        const int c0 = sm.woff[lw] - base;
-                        const int nrec = lane_on ? sm.woff[hw] - sm.woff[lw] : 0;
-                        if (BWD) {
-                            if (nrec > 0) scatter_list<V>(go, on, sm.roff + c0, sm.rw + c0, nrec, p.rstep, gfv);
-                        } else {
-                            gather_list<V, BF16, kWide>(acc, roff_s + 4 * c0, rw_s + 8 * c0, nrec, (unsigned)p.rstep, featv);
-                        }
-                        pos = upto;
-                    }
-                    round_end = s + 1;
-                }
+                } while (more);
                 if (BWD) continue;
 
                 // ---- the one store of every output vector
