@@ -157,7 +157,8 @@ flashbev_status flashbev_sampling_vt(const flashbev_vt_params *p, void *stream);
 
 /* Device scratch the operator can use beyond its inputs and outputs.  0 for channels-last (NHWC)
  * tensors with rows of whole 16-byte vectors (Sec. 3.3.1: all intermediates live in registers / on
- * chip).  For NCHW tensors with such rows: the size of a channels-last copy of the features; for
+ * chip).  For NCHW tensors: the size of a channels-last copy of the features, its rows padded to whole
+ * vectors (0 for channel counts that need padding on grids of fewer than 12288 bins B*X*Y*Z); for
  * channels-last tensors with other channel counts: the size of a copy with the rows padded to whole
  * vectors.  `workspace` may lend it to the call (optional; see the field). */
 size_t flashbev_workspace_bytes(const flashbev_vt_params *p);

@@ -630,27 +630,27 @@ __global__ void __launch_bounds__(128, V <= 2 ? 5 : 3) sca_kernel(const ScaParam
 }
 
 // ------------------------------------------------------------------------------------------
-// Channel-planar features [planes][C][HW] -> channels last [planes][HW][C] (T: 2- or 4-byte elements, C a multiple of the E
-// elements of 16 bytes).  Bound by memory: a thread reads 16 bytes of E channel rows, transposes the E x E block in registers
+// Channel-planar features [planes][C][HW] -> channels last [planes][HW][Cpad] (T: 2- or 4-byte elements, Cpad: C rounded up to the
+// E elements of 16 bytes, the tail zero).  Bound by memory: a thread reads 16 bytes of E channel rows, transposes the E x E block in registers
 // (bf16: 32 byte permutes) and writes 16 bytes of E texels.  A warp covers 4 E channels x 8 E texels, so it reads whole
 // 128-byte lines and writes 64-byte pieces.  ALIGNED: HW is a multiple of E and the base is 16-byte aligned; otherwise the rows
 // are read element by element (they hit L1).  Measured on 6 x 128 x 64 x 176 bf16 (17 MB): 25 us with a 32 x 32 shared-memory
 // tile of 2-byte accesses, 7.6 us now.
 template <typename T, bool ALIGNED>
-__global__ void __launch_bounds__(256) nchw_to_nhwc_kernel(const T *__restrict__ in, T *__restrict__ out, int C, int HW)
+__global__ void __launch_bounds__(256) nchw_to_nhwc_kernel(const T *__restrict__ in, T *__restrict__ out, int C, int Cpad, int HW)
 {
     constexpr int E = 16 / (int)sizeof(T);
     asm volatile("griddepcontrol.launch_dependents;");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int hw0 = (blockIdx.x * 8 + warp) * (8 * E) + (lane >> 2) * E, c0 = (blockIdx.y * 4 + (lane & 3)) * E;
-    if (hw0 >= HW || c0 >= C) return;
+    if (hw0 >= HW || c0 >= Cpad) return;
     const T *src = in + ((size_t)blockIdx.z * C + c0) * HW + hw0;
-    T *dst = out + ((size_t)blockIdx.z * HW + hw0) * C + c0;
+    T *dst = out + ((size_t)blockIdx.z * HW + hw0) * Cpad + c0;
     uint32_t r[E][4];
     if (ALIGNED) {
 #pragma unroll
         for (int i = 0; i < E; ++i) {
-            const uint4 v = __ldcs(reinterpret_cast<const uint4 *>(src + (size_t)i * HW));
+            const uint4 v = c0 + i < C ? __ldcs(reinterpret_cast<const uint4 *>(src + (size_t)i * HW)) : make_uint4(0u, 0u, 0u, 0u);
             r[i][0] = v.x, r[i][1] = v.y, r[i][2] = v.z, r[i][3] = v.w;
         }
     } else {
@@ -658,7 +658,7 @@ __global__ void __launch_bounds__(256) nchw_to_nhwc_kernel(const T *__restrict__
         for (int i = 0; i < E; ++i) {
             uint32_t e[E];
 #pragma unroll
-            for (int j = 0; j < E; ++j) e[j] = hw0 + j < HW ? (uint32_t)*reinterpret_cast<const typename std::conditional<sizeof(T) == 2, uint16_t, uint32_t>::type *>(src + (size_t)i * HW + j) : 0u;
+            for (int j = 0; j < E; ++j) e[j] = c0 + i < C && hw0 + j < HW ? (uint32_t)*reinterpret_cast<const typename std::conditional<sizeof(T) == 2, uint16_t, uint32_t>::type *>(src + (size_t)i * HW + j) : 0u;
 #pragma unroll
             for (int j = 0; j < 4; ++j) r[i][j] = sizeof(T) == 2 ? e[(2 * j) % E] | (e[(2 * j + 1) % E] << 16) : e[j % E];
         }
@@ -674,7 +674,7 @@ __global__ void __launch_bounds__(256) nchw_to_nhwc_kernel(const T *__restrict__
         } else {
             v = make_uint4(r[0][j % 4], r[1][j % 4], r[2][j % 4], r[3][j % 4]);
         }
-        *reinterpret_cast<uint4 *>(dst + (size_t)j * C) = v;
+        *reinterpret_cast<uint4 *>(dst + (size_t)j * Cpad) = v;
     }
 }
 
@@ -856,11 +856,25 @@ bool tiled_applicable(const flashbev_vt_params *p)
     return tiled_shape_ok(p);
 }
 
-// Bytes of the channels-last copy of NCHW features (0: the shape cannot take the tiled kernel).
+// Channels rounded up to whole 16-byte vectors.
+int padded_channels(const flashbev_vt_params *p)
+{
+    const int vec = p->feat_dtype == FLASHBEV_F32 ? 4 : 8;
+    return (p->C + vec - 1) / vec * vec;
+}
+
+// Bytes of the channels-last copy of NCHW features (0: not worth it, or the shape cannot take the tiled kernel).  Channel
+// counts that are not whole vectors are padded in the copy.  Grids of fewer than 12 K bins keep the generic kernel for those (one
+// launch, no scratch to find for callers of the smallest grids; 30-45 us either way of the line).  Measured with six 29 x 77
+// maps of 97 bf16 channels: 53 -> 20 us on 64 x 64 x 8 bins, 485 -> 62 us on 200 x 200 x 16.
 size_t nchw_copy_bytes(const flashbev_vt_params *p)
 {
-    if (p->layout != FLASHBEV_NCHW || !tiled_shape_ok(p)) return 0;
-    return (size_t)p->B * p->N * p->feat_h * p->feat_w * p->C * (p->feat_dtype == FLASHBEV_F32 ? 4 : 2);
+    if (p->layout != FLASHBEV_NCHW) return 0;
+    flashbev_vt_params q = copy_params(p);
+    q.C = padded_channels(p);
+    if (q.C != p->C && (double)p->B * p->X * p->Y * p->Z < 12288.0) return 0;
+    if (!tiled_shape_ok(&q)) return 0;
+    return (size_t)p->B * p->N * p->feat_h * p->feat_w * q.C * (p->feat_dtype == FLASHBEV_F32 ? 4 : 2);
 }
 
 // NCHW tensors with a workspace that holds the channels-last copy: transposing copy, then the tiled kernel.
@@ -869,14 +883,7 @@ bool nchw_tiled_applicable(const flashbev_vt_params *p)
     if (p->struct_size < sizeof(flashbev_vt_params) || !p->workspace) return false;
     const size_t need = nchw_copy_bytes(p);
     return need && p->workspace_bytes >= need && (uintptr_t)p->workspace % 16 == 0 &&
-           (long long)p->B * p->N <= 65535 && (p->C + 31) / 32 <= 65535;
-}
-
-// Channels-last tensors whose rows are not whole 16-byte vectors: channels rounded up to the next whole vector.
-int padded_channels(const flashbev_vt_params *p)
-{
-    const int vec = p->feat_dtype == FLASHBEV_F32 ? 4 : 8;
-    return (p->C + vec - 1) / vec * vec;
+           (long long)p->B * p->N <= 65535 && (p->C + 15) / 16 <= 65535;
 }
 
 // Bytes of the padded copy of such features (0: not that case, or the padded shape cannot take the tiled kernel).
@@ -1063,8 +1070,8 @@ flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V,
     return FLASHBEV_OK;
 }
 
-// scalar_out: 0 vector stores into channels-last rows; 1 planar output [B][C][X][Y]; 2 channels-last rows of out_c
-// channels (the kernel's own C is padded)
+// scalar_out: 0 vector stores into channels-last rows; 1 planar output [B][out_c][X][Y]; 2 channels-last rows of out_c
+// channels (the kernel's own C may be padded)
 flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, bool accumulate = false, int scalar_out = 0,
                              int out_c = 0)
 {
@@ -1077,7 +1084,7 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
     k.out_nchw = scalar_out != 0;
     {
         const size_t plane = (size_t)p->X * p->Y;
-        if (scalar_out == 1) k.out_c = p->C, k.out_bs = plane * p->C, k.out_cells = 1, k.out_chs = plane;
+        if (scalar_out == 1) k.out_c = out_c, k.out_bs = plane * out_c, k.out_cells = 1, k.out_chs = plane;
         if (scalar_out == 2) k.out_c = out_c, k.out_bs = plane * out_c, k.out_cells = out_c, k.out_chs = 1;
     }
     k.pdl = getenv("FLASHBEV_NO_PDL") ? 0 : 1;
@@ -1104,6 +1111,7 @@ flashbev_status launch_nchw_tiled(const flashbev_vt_params *p, cudaStream_t stre
     flashbev_vt_params q = *p;
     q.features = p->workspace;
     q.layout = FLASHBEV_NHWC;
+    q.C = padded_channels(p);
     q.tune[3] = (q.tune[3] & ~0xf) | 4;  // the planar-output instances are built for 4 warps per CTA
     {   // configure first: nothing is enqueued for a shape the tiled kernel cannot take
         KParams k;
@@ -1116,15 +1124,15 @@ flashbev_status launch_nchw_tiled(const flashbev_vt_params *p, cudaStream_t stre
     const int HW = p->feat_h * p->feat_w;
     const int E = p->feat_dtype == FLASHBEV_BF16 ? 8 : 4;
     const bool aligned = HW % E == 0 && (uintptr_t)p->features % 16 == 0;
-    const dim3 grid((unsigned)((HW + 64 * E - 1) / (64 * E)), (unsigned)((p->C + 4 * E - 1) / (4 * E)), (unsigned)(p->B * p->N));
+    const dim3 grid((unsigned)((HW + 64 * E - 1) / (64 * E)), (unsigned)((q.C + 4 * E - 1) / (4 * E)), (unsigned)(p->B * p->N));
     auto copy = [&](auto kernel, auto *elem) {
         using T = typename std::remove_pointer<decltype(elem)>::type;
-        kernel<<<grid, dim3(256), 0, stream>>>(static_cast<const T *>(p->features), static_cast<T *>(p->workspace), p->C, HW);
+        kernel<<<grid, dim3(256), 0, stream>>>(static_cast<const T *>(p->features), static_cast<T *>(p->workspace), p->C, q.C, HW);
     };
     if (E == 8) aligned ? copy(nchw_to_nhwc_kernel<uint16_t, true>, (uint16_t *)nullptr) : copy(nchw_to_nhwc_kernel<uint16_t, false>, (uint16_t *)nullptr);
     else aligned ? copy(nchw_to_nhwc_kernel<float, true>, (float *)nullptr) : copy(nchw_to_nhwc_kernel<float, false>, (float *)nullptr);
     if (cudaGetLastError() != cudaSuccess) return FLASHBEV_CUDA_ERROR;
-    const flashbev_status st = launch_tiled(&q, stream, accumulate, 1);
+    const flashbev_status st = launch_tiled(&q, stream, accumulate, 1, p->C);
     if (st == FLASHBEV_OK) t_last_kernel = p->feat_dtype == FLASHBEV_BF16 ? "tiled_bf16_nchw" : "tiled_f32_nchw";
     return st;
 }
