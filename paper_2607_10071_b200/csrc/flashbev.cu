@@ -376,8 +376,10 @@ __global__ void __launch_bounds__(256) vt_per_output_nchw_kernel(const KParams p
 //      in shared memory;
 //   2. for every camera that sees the query, the lanes turn (head, level, point) triples -- read with
 //      coalesced streaming loads in the order the offsets and weights are stored -- into tap records
-//      {4 value indices, 4 weights} in shared memory: attention weight x bilinear weight, out-of-map taps
-//      clamped to an in-map address with weight 0 (zero padding without predicates);
+//      {index of the upper left tap, 4 weights} in shared memory: attention weight x bilinear weight; the 2 x 2 block
+//      of taps is moved inside the map and the taps outside of it weigh 0 (zero padding without predicates).
+//      The other three taps are one texel and one row further (20 bytes per record: with all four indices, 32 bytes,
+//      the records were a third of the L1 data pipe's wavefronts, the unit that bounds this kernel: @@M@@);
 //   3. the lanes of a head (head_dim / 4 lanes, 16 bytes of the head's channels each) walk the head's
 //      records: four 128-bit loads and packed fp32 FMAs per record.
 // No per-camera, BEV-shaped tensor (reference points, masks, sampling locations) ever exists in memory.
@@ -400,13 +402,13 @@ struct ScaParams {
     int Hl[kScaMaxLevels], Wl[kScaMaxLevels], lvl0[kScaMaxLevels];
 };
 
-// Shared memory of one warp: reference points, visibility masks, tap records (16 + 16 bytes each), the
+// Shared memory of one warp: reference points, visibility masks, tap records (16 + 4 bytes each), the
 // texel positions of the references of one camera (16 bytes per height x level) and two staging buffers
 // for the (offset, weight) pairs of a chunk (8 + 4 bytes per head x level x point).
 __host__ __device__ inline size_t sca_warp_smem(int N, int Zref, int heads, int pitch, int items, int L)
 {
     return (size_t)N * Zref * sizeof(double2) + (((size_t)N * sizeof(uint32_t) + 15) & ~(size_t)15) +
-           (size_t)heads * pitch * 32 + (size_t)Zref * L * 16 + 2 * (((size_t)items * 12 + 15) & ~(size_t)15);
+           (((size_t)heads * pitch * 20 + 15) & ~(size_t)15) + (size_t)Zref * L * 16 + 2 * (((size_t)items * 12 + 15) & ~(size_t)15);
 }
 
 __device__ __forceinline__ void cp_async_4(void *dst, const void *src)
@@ -451,9 +453,10 @@ __global__ void __launch_bounds__(128, V <= 2 ? 5 : 3) sca_kernel(const ScaParam
                           warp * sca_warp_smem(p.N, p.Zref, p.heads, p.pitch, max_items, p.L);
     double2 *ref = reinterpret_cast<double2 *>(mine);
     uint32_t *vm = reinterpret_cast<uint32_t *>(mine + (size_t)nref * sizeof(double2));
-    uint4 *rec_i = reinterpret_cast<uint4 *>(mine + (size_t)nref * sizeof(double2) + (((size_t)p.N * 4 + 15) & ~(size_t)15));
-    float4 *rec_w = reinterpret_cast<float4 *>(rec_i + cap);
-    int4 *base_tab = reinterpret_cast<int4 *>(rec_w + cap);                       // [Zref][L]: texel position of a reference
+    float4 *rec_w = reinterpret_cast<float4 *>(mine + (size_t)nref * sizeof(double2) + (((size_t)p.N * 4 + 15) & ~(size_t)15));
+    uint32_t *rec_i = reinterpret_cast<uint32_t *>(rec_w + cap);
+    // [Zref][L]: texel position of a reference
+    int4 *base_tab = reinterpret_cast<int4 *>(reinterpret_cast<unsigned char *>(rec_w) + (((size_t)cap * 20 + 15) & ~(size_t)15));
     unsigned char *stage = reinterpret_cast<unsigned char *>(base_tab + p.Zref * p.L);  // [2][offsets | weights]
 
     const size_t qrow = ((size_t)b * Q + q) * (size_t)(p.heads * p.L);  // first (head, level) row of the query
@@ -563,32 +566,24 @@ __global__ void __launch_bounds__(128, V <= 2 ? 5 : 3) sca_kernel(const ScaParam
                 const float flx = floorf(sx), fly = floorf(sy);
                 const float tx = sx - flx, ty = sy - fly;
                 const int x0 = bs.x + (int)flx, y0 = bs.y + (int)fly;
-                const bool inx0 = (unsigned)x0 < (unsigned)Wl, inx1 = (unsigned)(x0 + 1) < (unsigned)Wl;
-                const bool iny0 = (unsigned)y0 < (unsigned)Hl, iny1 = (unsigned)(y0 + 1) < (unsigned)Hl;
-                const int xa = min(max(x0, 0), Wl - 1), xb = min(max(x0 + 1, 0), Wl - 1);
-                const int ya = min(max(y0, 0), Hl - 1), yb = min(max(y0 + 1, 0), Hl - 1);
-                const float wx0 = a * (1.f - tx), wx1 = a * tx;
-                float4 w;
-                w.x = inx0 && iny0 ? wx0 * (1.f - ty) : 0.f;
-                w.y = inx1 && iny0 ? wx1 * (1.f - ty) : 0.f;
-                w.z = inx0 && iny1 ? wx0 * ty : 0.f;
-                w.w = inx1 && iny1 ? wx1 * ty : 0.f;
-                const uint32_t hoff = (uint32_t)(h * p.lph);
-                const uint32_t ra = (uint32_t)(p.lvl0[l] + ya * Wl), rb = (uint32_t)(p.lvl0[l] + yb * Wl);
-                uint4 ti;
-                ti.x = (ra + xa) * D4 + hoff;
-                ti.y = (ra + xb) * D4 + hoff;
-                ti.z = (rb + xa) * D4 + hoff;
-                ti.w = (rb + xb) * D4 + hoff;
+                // the 2 x 2 block at (xc, yc) inside the map, the weights of its columns and rows
+                const int xc = min(max(x0, 0), max(Wl - 2, 0)), yc = min(max(y0, 0), max(Hl - 2, 0));
+                const float wx0 = a * (x0 == xc ? 1.f - tx : (x0 + 1 == xc ? tx : 0.f));
+                const float wx1 = a * (x0 == xc ? (Wl > 1 ? tx : 0.f) : (x0 == xc + 1 && Wl > 1 ? 1.f - tx : 0.f));
+                const float wy0 = y0 == yc ? 1.f - ty : (y0 + 1 == yc ? ty : 0.f);
+                const float wy1 = y0 == yc ? (Hl > 1 ? ty : 0.f) : (y0 == yc + 1 && Hl > 1 ? 1.f - ty : 0.f);
+                const float4 w = make_float4(wx0 * wy0, wx1 * wy0, wx0 * wy1, wx1 * wy1);
+                const uint32_t ti = (uint32_t)(p.lvl0[l] + yc * Wl + xc) * D4 + (uint32_t)(h * p.lph);
                 rec_i[i + h] = ti;  // = head * pitch + level * Pc + point
                 rec_w[i + h] = w;
             }
             __syncwarp();
             // ---- phase 3: gather, every lane over the records of its heads
             for (int l = 0; l < p.L; ++l) {
+                const uint32_t right = p.Wl[l] > 1 ? D4 : 0, below = p.Hl[l] > 1 ? p.Wl[l] * D4 : 0;
                 for (uint32_t m = vis; m; m &= m - 1u) {
                     const int slot = l * p.Pc + __ffs(m) - 1;
-                    uint4 ti[V];
+                    uint32_t ti[V];
                     float4 tw[V];
                     uint4 s[V][4];
 #pragma unroll
@@ -599,10 +594,10 @@ __global__ void __launch_bounds__(128, V <= 2 ? 5 : 3) sca_kernel(const ScaParam
 #pragma unroll
                     for (int v = 0; v < V; ++v) {
                         if (!on[v]) continue;
-                        s[v][0] = __ldg(vcam + ti[v].x);
-                        s[v][1] = __ldg(vcam + ti[v].y);
-                        s[v][2] = __ldg(vcam + ti[v].z);
-                        s[v][3] = __ldg(vcam + ti[v].w);
+                        s[v][0] = __ldg(vec_at(vcam, ti[v]));
+                        s[v][1] = __ldg(vec_at(vcam, ti[v] + right));
+                        s[v][2] = __ldg(vec_at(vcam, ti[v] + below));
+                        s[v][3] = __ldg(vec_at(vcam, ti[v] + below + right));
                     }
 #pragma unroll
                     for (int v = 0; v < V; ++v) {
