@@ -425,10 +425,11 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // EVEN: every lane has a head in every pass (heads = V * heads per pass, 32 lanes all used)
-// Seven CTAs per SM (72 registers) for up to two vectors per lane: the gather waits on L2 most of the time.  N = 6, C = 256,
-// 200 x 200, P = 8: fp32 394 / 358 / 355 / 350 / 432 us at 4 / 5 / 6 / 7 / 8, bf16 309 / 309 / 282 / 270 / 378.
+// bf16 takes seven CTAs per SM (72 registers): the gather waits on L2 most of the time.  N = 6, C = 256, 200 x 200, P = 8:
+// 309 / 282 / 274 / 378 us at 5 / 6 / 7 / 8.  fp32 moves twice the bytes through L1 and gains nothing (363 / 362 / 364 us),
+// a 120 x 90 grid loses 3 %: five.
 template <int V, bool EVEN, bool BF16>
-__global__ void __launch_bounds__(128, V <= 2 ? 7 : 3) sca_kernel(const ScaParams p)
+__global__ void __launch_bounds__(128, V <= 2 ? (BF16 ? 7 : 5) : 3) sca_kernel(const ScaParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr unsigned FULL = 0xffffffffu;
