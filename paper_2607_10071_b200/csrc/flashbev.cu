@@ -59,7 +59,11 @@ struct KParams {
     int wx, wy;                 // sub-block size in cells (x, y)
     int sbx, sby, sbn;          // sub-blocks per super-block (x, y, total)
     int ct;                     // cells per super-block (<= 32)
-    float inv_n;                // 1 / N
+    float inv_n, inv_z;         // 1 / N, 1 / Z
+    int inv_sby, inv_wy;        // ceil(65536 / sby), ceil(65536 / wy)
+    int band_shift;             // log2 of the band height
+    unsigned band_mul;          // n / (super-blocks of a band) = n * band_mul >> band_mul_shift for n < 2^31
+    int band_mul_shift;
     int blocks_x, blocks_y;     // super-blocks per batch element
     int band, reps;             // super-block order: bands of `band` rows; super-blocks per warp
     int nbands, centre_out;     // number of bands; visit them from the middle of the grid outwards
@@ -954,7 +958,7 @@ flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V,
     k.vecs = p->C * elem / 16;
     k.rstep = p->feat_w > 1 ? k.vecs : 0;
     k.nvec_cam = p->N * p->feat_h * p->feat_w * k.vecs;  // < 2^31: tiled_applicable
-    k.inv_n = 1.0f / (float)p->N;
+    k.inv_n = 1.0f / (float)p->N, k.inv_z = 1.0f / (float)p->Z;
 
     // channel mapping: V vectors per lane, g lanes per cell
     V = p->tune[0];
@@ -1042,6 +1046,15 @@ flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V,
 
     const long long bands = (k.blocks_x + k.band - 1) / k.band;
     k.nbands = (int)bands;
+    // (a warp decodes its task once: the integer divisions were about 100 instructions of its 700 before the first column)
+    k.inv_sby = (65536 + sby - 1) / sby, k.inv_wy = (65536 + k.wy - 1) / k.wy;
+    for (k.band_shift = 0; (1 << k.band_shift) < k.band; ++k.band_shift) {}
+    {
+        const unsigned long long d = (unsigned long long)k.band * (unsigned)k.blocks_y;  // the ids are below 2^31
+        int sh = 0;
+        while ((1ull << sh) < d) ++sh;
+        k.band_mul_shift = 31 + sh, k.band_mul = (unsigned)((1ull << k.band_mul_shift) / d + 1);
+    }
     k.centre_out = !((p->tune[3] >> 28) & 1);
     const long long sbs = bands * k.band * k.blocks_y;  // super-blocks in visiting order (those past the grid's edge do nothing)
     // the tail of the order is split into single sub-blocks: about one warp's worth per resident warp slot

@@ -749,7 +749,7 @@ __device__ __forceinline__ int build_columns(const KParams &p, WarpCtx cx, int j
     }
     if (p.reduce == FLASHBEV_REDUCE_CAMERA_MEAN_Z_SUM) {
         for (int i = c_lo * p.Z + lane; i < c_hi * p.Z; i += 32) {
-            const int c = i / p.Z, k = i - c * p.Z;
+            const int c = (int)(((float)i + 0.5f) * p.inv_z), k = i - c * p.Z;  // (i < 2^20)
             int dn = 0;
             for (int j = sm.cfirst[c] - jb; j < sm.cfirst[c + 1] - jb; ++j) {
                 const int kk = sm.col[j].kk;
@@ -826,9 +826,9 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
     for (int c = tid; c < kMaxCt; c += THREADS) {
         int v = 0;
         if (c < p.ct) {
-            const int s = c / p.cpw, j = c - s * p.cpw;  // sub-block, cell inside it
-            const int si = s / p.sby, sj = s - si * p.sby;
-            const int jx = j / p.wy, jy = j - jx * p.wy;
+            const int s = c * p.inv_cpw >> 16, j = c - s * p.cpw;  // sub-block, cell inside it
+            const int si = s * p.inv_sby >> 16, sj = s - si * p.sby;
+            const int jx = j * p.inv_wy >> 16, jy = j - jx * p.wy;
             v = (si * p.wx + jx) | ((sj * p.wy + jy) << 8);
         }
         celltab[c] = v;
@@ -871,14 +871,13 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
             id = p.whole_tasks + q, s_begin = k - q * p.sbn, s_end = s_begin + 1;
         }
         if (id >= p.total_sbs) continue;  // (padding warps of the last CTA; warp-uniform)
-        const int per_band = p.band * p.blocks_y;
-        int bandi = id / per_band;
-        const int rem = id - bandi * per_band;
+        int bandi = (int)((unsigned long long)(unsigned)id * p.band_mul >> p.band_mul_shift);  // id / (super-blocks of a band)
+        const int rem = id - bandi * (p.blocks_y << p.band_shift);
         if (p.centre_out) {  // bands from the middle of the grid outwards: the cells around the ego write the most records
             const int half = (bandi + 1) >> 1;
             bandi = ((p.nbands - 1) >> 1) + ((bandi & 1) ? half : -half);
         }
-        const int by = rem / p.band, bx = bandi * p.band + (rem - by * p.band);
+        const int by = rem >> p.band_shift, bx = (bandi << p.band_shift) + (rem - (by << p.band_shift));
         if ((unsigned)bx >= (unsigned)p.blocks_x || (unsigned)by >= (unsigned)p.blocks_y) continue;  // past the grid's edge; warp-uniform
         const int ix0 = bx * (p.sbx * p.wx), iy0 = by * (p.sby * p.wy);
 
