@@ -939,17 +939,17 @@ cudaError_t launch_tiled_warps(int warps, const KParams &k, dim3 grid, size_t sm
         case 8: return launch_tiled_inst<V, BF16, 8, false>(k, grid, smem, stream);
         default:
             if (k.out_nchw) {  // (planar output: instances for 4 warps per CTA only)
-                if (V >= 2 && k.wide) return launch_tiled_inst<V, BF16, 4, false, (V >= 2), true>(k, grid, smem, stream);
+                if (V % 2 == 0 && k.wide) return launch_tiled_inst<V, BF16, 4, false, (V % 2 == 0), true>(k, grid, smem, stream);
                 return launch_tiled_inst<V, BF16, 4, false, false, true>(k, grid, smem, stream);
             }
-            if (V >= 2 && k.wide) return launch_tiled_inst<V, BF16, 4, false, (V >= 2)>(k, grid, smem, stream);
+            if (V % 2 == 0 && k.wide) return launch_tiled_inst<V, BF16, 4, false, (V % 2 == 0)>(k, grid, smem, stream);
             return launch_tiled_inst<V, BF16, 4, false>(k, grid, smem, stream);
     }
 }
 
 // Chooses the channel mapping, super-block shape, run length, list size and grid of the tiled kernel.
 flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V, int &warps, dim3 &grid, size_t &smem,
-                                bool accumulate = false)
+                                bool accumulate = false, bool backward = false)
 {
     k = base_params(p, accumulate);
     const bool bf16 = p->feat_dtype == FLASHBEV_BF16;
@@ -965,8 +965,12 @@ flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V,
     int g = p->tune[1];
     if (!(V == 1 || V == 2 || V == 4) || g < 1 || g > 32) V = 0, g = 0;
     if (!V) {
-        // (measured) up to 8 vectors per texel: one per lane; up to 32: two adjacent ones per lane; beyond: four.
+        // (measured) up to 8 vectors per texel: one per lane; up to 32: two adjacent ones per lane; beyond: four.  fp32 forward:
+        // three where two leave a quarter of the lanes without a cell (21-24 vectors: two cells of 12 lanes) or four halve the
+        // residency (33-48).  200 x 200 x 8: C = 96 44.2 -> 38.2 us, 84 47.9 -> 45.8, 192 69.6 -> 61.9, 144 69.7 -> 61.1.  Not
+        // bf16, which loses its 256-bit loads (C = 192: 60.8 -> 59.2, small grids 37.5 -> 38.3), nor the backward (97 -> 103).
         if (k.vecs <= 8) V = 1, g = k.vecs;
+        else if (!bf16 && !backward && ((k.vecs >= 21 && k.vecs <= 24) || (k.vecs >= 33 && k.vecs <= 48))) V = 3, g = (k.vecs + 2) / 3;
         else if (k.vecs <= 32) V = (k.vecs % 2 == 0 || k.vecs > 16) ? 2 : 1, g = (k.vecs + V - 1) / V;
         else V = 4, g = (k.vecs + 3) / 4;
         if (g > 32) g = 32;
@@ -1102,8 +1106,8 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
     k.pdl = getenv("FLASHBEV_NO_PDL") ? 0 : 1;
     const bool bf16 = p->feat_dtype == FLASHBEV_BF16;
     cudaError_t e;
-    static const char *const names[2][3] = {{"tiled_f32_v1", "tiled_f32_v2", "tiled_f32_v4"},
-                                            {"tiled_bf16_v1", "tiled_bf16_v2", "tiled_bf16_v4"}};
+    static const char *const names[2][4] = {{"tiled_f32_v1", "tiled_f32_v2", "tiled_f32_v3", "tiled_f32_v4"},
+                                            {"tiled_bf16_v1", "tiled_bf16_v2", "", "tiled_bf16_v4"}};
     if (bf16) {
         if (V == 1) e = launch_tiled_warps<1, true>(warps, k, grid, smem, stream);
         else if (V == 2) e = launch_tiled_warps<2, true>(warps, k, grid, smem, stream);
@@ -1111,9 +1115,10 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
     } else {
         if (V == 1) e = launch_tiled_warps<1, false>(warps, k, grid, smem, stream);
         else if (V == 2) e = launch_tiled_warps<2, false>(warps, k, grid, smem, stream);
+        else if (V == 3) e = launch_tiled_warps<3, false>(warps, k, grid, smem, stream);
         else e = launch_tiled_warps<4, false>(warps, k, grid, smem, stream);
     }
-    t_last_kernel = names[bf16 ? 1 : 0][V == 1 ? 0 : (V == 2 ? 1 : 2)];
+    t_last_kernel = names[bf16 ? 1 : 0][V - 1];
     return e == cudaSuccess ? FLASHBEV_OK : FLASHBEV_CUDA_ERROR;
 }
 
@@ -1345,7 +1350,7 @@ flashbev_status flashbev_sampling_vt_backward(const flashbev_vt_backward_params 
         if (!(p.tune[3] & 0xff0)) p.tune[3] |= (1 << 4) | (2 << 8);
         if (!(p.tune[3] & 0xc0000)) p.tune[3] |= 0x40000;
     }
-    if ((st = configure_tiled(&p, k, V, warps, grid, smem)) != FLASHBEV_OK) return st;
+    if ((st = configure_tiled(&p, k, V, warps, grid, smem, false, true)) != FLASHBEV_OK) return st;
     k.feat = nullptr, k.out = nullptr, k.count_out = nullptr;
     k.gout = q->grad_out, k.gfeat = q->grad_features;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);

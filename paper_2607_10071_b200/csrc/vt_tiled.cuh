@@ -838,7 +838,7 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
     // ---- gather role of this lane inside a sub-block
     const int cg = (lane * p.inv_g) >> 16, gl = lane - cg * p.g;  // lane / g
     const bool role = cg < p.cpw;
-    constexpr bool kWide = WIDE && V >= 2 && !BWD;
+    constexpr bool kWide = WIDE && V % 2 == 0 && !BWD;
     const int vstep = kWide ? 1 : p.g;  // distance between the lane's channel vectors
     const int vec0 = kWide ? (blockIdx.y * p.g + gl) * V : blockIdx.y * (p.g * V) + gl;  // the lane's first vector
     // channel vectors past the end of the row (ragged last channel block) re-read vector 0, never stored

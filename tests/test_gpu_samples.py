@@ -52,3 +52,15 @@ def test_feature_copies(layout, dtype, C, feat):
     assert fb.flashbev_last_kernel_name().endswith("nchw" if layout == fb.NCHW else "padded")
     out = out.permute(0, 2, 3, 1) if layout == fb.NCHW else out
     assert torch.equal(out, ref)
+
+
+@pytest.mark.parametrize("C", [80, 84, 88, 96, 100, 128, 132, 144, 160, 192, 196])
+def test_vectors_per_lane(oracle, C):
+    """Channel counts on both sides of every change in the number of channel vectors per lane (fp32)."""
+    inp = inputs(6, True, C=C)
+    w = inp.workload
+    for reduce in (0, 1):
+        ref = oracle.sampling_vt(inp.features, inp.lidar2img, w.img_hw, w.bev_range, w.grid, reduce)
+        out, cnt, _ = parity.run_gpu(inp, reduce, fb.KERNEL_TILED)
+        parity.assert_parity(w, ref, out, cnt, f"[C={C} reduce={reduce}]", check_fraction=False)
+    check_backward(oracle, w, inp.lidar2img, 0)
