@@ -10,8 +10,10 @@
 #include <ATen/ops/empty.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <exception>
 #include <vector>
 
 #include "flashbev.h"
@@ -128,7 +130,8 @@ void need_args(Py_ssize_t n, Py_ssize_t want)
     throw Bad();
 }
 
-// `body` with C++ exceptions turned into Python errors
+// `body` with C++ exceptions turned into the Python errors that PyTorch's own functions raise for them: a failed allocation is
+// torch.OutOfMemoryError (callers catch it, free memory and try again), a missing dimension IndexError.
 template <typename F>
 PyObject *guarded(F body)
 {
@@ -136,8 +139,8 @@ PyObject *guarded(F body)
         return body();
     } catch (const Bad &) {
         return nullptr;
-    } catch (const std::exception &e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
+    } catch (...) {
+        torch::translate_exception_to_python(std::current_exception());
         return nullptr;
     }
 }
