@@ -47,14 +47,36 @@ int64_t integer(PyObject *o)
     return v;
 }
 
-int32_t integer32(PyObject *o)
+int32_t narrow(int64_t v)
 {
-    const int64_t v = integer(o);
     if (v != (int32_t)v) {
         PyErr_SetString(PyExc_OverflowError, "argument does not fit 32 bits");
         throw Bad();
     }
     return (int32_t)v;
+}
+
+int32_t integer32(PyObject *o) { return narrow(integer(o)); }
+
+// int(o): numbers of any kind, cut to whole ones
+int32_t cut_integer32(PyObject *o)
+{
+    PyObject *i = PyNumber_Long(o);
+    if (!i) throw Bad();
+    const long long v = PyLong_AsLongLong(i);
+    Py_DECREF(i);
+    if (v == -1 && PyErr_Occurred()) throw Bad();
+    return narrow(v);
+}
+
+// float(o)
+double real(PyObject *o)
+{
+    PyObject *f = PyNumber_Float(o);
+    if (!f) throw Bad();
+    const double v = PyFloat_AS_DOUBLE(f);
+    Py_DECREF(f);
+    return v;
 }
 
 // The n items of a sequence, handed to `f(index, item)`
@@ -82,10 +104,7 @@ void geometry(P &p, PyObject *img_hw, PyObject *bev_range)
     items(img_hw, 2, "img_hw must be (height, width)", [&](Py_ssize_t i, PyObject *v) { hw[i] = integer32(v); });
     p.img_h = hw[0], p.img_w = hw[1];
     double r[6];
-    items(bev_range, 6, "bev_range must have six numbers", [&](Py_ssize_t i, PyObject *v) {
-        r[i] = PyFloat_AsDouble(v);
-        if (r[i] == -1.0 && PyErr_Occurred()) throw Bad();
-    });
+    items(bev_range, 6, "bev_range must have six numbers", [&](Py_ssize_t i, PyObject *v) { r[i] = real(v); });
     p.x_min = r[0], p.x_max = r[1], p.y_min = r[2], p.y_max = r[3], p.z_min = r[4], p.z_max = r[5];
 }
 
@@ -95,7 +114,7 @@ void tune(int32_t (&t)[4], PyObject *o)
     if (!seq) throw Bad();
     try {
         if (PySequence_Fast_GET_SIZE(seq) > 4) value_error("tune has at most four entries");
-        for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(seq); ++i) t[i] = integer32(PySequence_Fast_GET_ITEM(seq, i));
+        for (Py_ssize_t i = 0; i < PySequence_Fast_GET_SIZE(seq); ++i) t[i] = cut_integer32(PySequence_Fast_GET_ITEM(seq, i));
     } catch (...) {
         Py_DECREF(seq);
         throw;
@@ -203,9 +222,15 @@ PyObject *py_sampling_vt_backward(PyObject *, PyObject *const *a, Py_ssize_t n)
         p.N = (int32_t)m.size(1);
         items(a[2], 2, "feat_hw must be (height, width)", [&](Py_ssize_t i, PyObject *v) { (i ? p.feat_w : p.feat_h) = integer32(v); });
         geometry(p, a[3], a[4]);
-        items(a[5], 3, "grid must be (X, Y, Z)", [&](Py_ssize_t i, PyObject *v) {
-            if (i == 2) p.Z = integer32(v);
-        });
+        PyObject *z = PySequence_GetItem(a[5], 2);  // X and Y are those of grad_out
+        if (!z) throw Bad();
+        try {
+            p.Z = integer32(z);
+        } catch (...) {
+            Py_DECREF(z);
+            throw;
+        }
+        Py_DECREF(z);
         p.reduce = integer32(a[6]);
         tune(p.tune, a[8]);
         const c10::cuda::CUDAGuard guard(g.device());
@@ -289,11 +314,15 @@ PyObject *py_sca(PyObject *, PyObject *const *a, Py_ssize_t n)
         p.L = (int32_t)w.size(3), p.P = (int32_t)w.size(4);
         const Py_ssize_t levels = PySequence_Size(a[1]);
         if (levels < 0) throw Bad();
-        if (levels < p.L) value_error("level_hw must have an entry per level");
-        std::vector<int32_t> hw(2 * (size_t)levels);
-        items(a[1], levels, "level_hw must be a sequence of (height, width)", [&](Py_ssize_t i, PyObject *l) {
-            items(l, 2, "level_hw must be a sequence of (height, width)", [&](Py_ssize_t j, PyObject *x) { hw[2 * i + j] = integer32(x); });
+        std::vector<int32_t> hw;  // (height, width) pairs, or the same numbers one after another
+        items(a[1], levels, "level_hw must be a sequence of (height, width)", [&](Py_ssize_t, PyObject *l) {
+            const auto put = [&](Py_ssize_t, PyObject *x) { hw.push_back(cut_integer32(x)); };
+            const bool row = PySequence_Check(l) && PySequence_Size(l) >= 0;
+            PyErr_Clear();  // (a number of an array type is a sequence without a length)
+            if (row) items(l, 2, "level_hw must be a sequence of (height, width)", put);
+            else put(0, l);
         });
+        if (hw.size() < 2 * (size_t)p.L) value_error("level_hw must have an entry per level");
         geometry(p, a[5], a[6]);
         items(a[7], 3, "grid must be (X, Y, Zref)", [&](Py_ssize_t i, PyObject *x) { (i == 0 ? p.X : (i == 1 ? p.Y : p.Zref)) = integer32(x); });
         const c10::cuda::CUDAGuard guard(v.device());
@@ -302,7 +331,7 @@ PyObject *py_sca(PyObject *, PyObject *const *a, Py_ssize_t n)
         p.offsets = static_cast<const float *>(o.data_ptr()), p.weights = static_cast<const float *>(w.data_ptr());
         p.out = static_cast<float *>(out.data_ptr());
         if (a[9] != Py_None) p.hits_out = static_cast<int32_t *>(tensor(a[9], "hits").data_ptr());
-        p.chunk_records = integer32(a[11]);
+        p.chunk_records = cut_integer32(a[11]);
         const flashbev_status st = flashbev_sca(&p, stream_of(a[10], v));
         return st == FLASHBEV_OK ? THPVariable_Wrap(std::move(out)) : status(st);
     });

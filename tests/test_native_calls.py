@@ -22,6 +22,35 @@ def test_rig_with_too_few_dimensions_is_an_index_error():
 
 
 @pytest.mark.gpu
+def test_numbers_are_converted_as_python_converts_them():
+    """bev_range by float(), hints by int(), level_hw as numpy casts it; the backward reads the height bins only from the grid."""
+    import numpy as np
+    import torch
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(3)
+    f = torch.randn((1, 2, 4, 6, 8), generator=gen, device=dev)
+    m = torch.eye(4, device=dev).expand(1, 2, 4, 4).contiguous()
+    m[:, :, :3, 3] = torch.tensor([24.0, 16.0, 4.0], device=dev)
+    img, r, grid = (32, 48), (-1.0, 1.0, -1.0, 1.0, -1.0, 1.0), (5, 6, 4)
+    want = fb.sampling_vt(f, m, img, r, grid)
+    assert float(want.abs().sum()) > 0
+    for ranges in (np.asarray(r, np.float32), torch.tensor(r), [str(v) for v in r]):
+        assert torch.equal(fb.sampling_vt(f, m, np.asarray(img), ranges, torch.tensor(grid), tune=(0.0, 0.0, np.float32(0), 0)), want)
+    grad = torch.randn((1, 5, 6, 8), generator=gen, device=dev)
+    back = fb.sampling_vt_backward(grad, m, (4, 6), img, r, grid)
+    assert torch.allclose(fb.sampling_vt_backward(grad, m, (4, 6), img, r, (None, None, 4, None)), back, rtol=1e-5, atol=1e-5)
+    value = torch.randn((1, 2, 30, 2, 8), generator=gen, device=dev)
+    off = torch.randn((1, 30, 2, 2, 4, 2), generator=gen, device=dev)
+    wts = torch.rand((1, 30, 2, 2, 4), generator=gen, device=dev)
+    att = fb.sca(value, ((4, 6), (2, 3)), m, off, wts, img, r, grid)
+    for hw in (np.array([[4, 6], [2, 3]]), np.array([4.0, 6.0, 2.0, 3.0]), torch.tensor([[4, 6], [2, 3]]), [4, 6, 2, 3, 9, 9],
+               torch.tensor([4.5, 6.0, 2.0, 3.0]), [[4, 6], np.array([2, 3])]):
+        assert torch.equal(fb.sca(value, hw, m, off, wts, img, r, grid, chunk_records=0.0), att)
+    with pytest.raises(ValueError):
+        fb.sca(value, [4, 6, 2], m, off, wts, img, r, grid)
+
+
+@pytest.mark.gpu
 def test_failed_allocation_is_an_out_of_memory_error_and_leaves_the_device_usable():
     import torch
     dev = torch.device("cuda:0")
