@@ -312,13 +312,13 @@ PyObject *py_sca(PyObject *, PyObject *const *a, Py_ssize_t n)
         p.value_dtype = v.scalar_type() == at::kFloat ? FLASHBEV_F32 : FLASHBEV_BF16;
         p.B = (int32_t)v.size(0), p.N = (int32_t)v.size(1), p.heads = (int32_t)v.size(3), p.head_dim = (int32_t)v.size(4);
         p.L = (int32_t)w.size(3), p.P = (int32_t)w.size(4);
-        const Py_ssize_t levels = PySequence_Size(a[1]);
+        const Py_ssize_t levels = PyObject_Size(a[1]);
         if (levels < 0) throw Bad();
         std::vector<int32_t> hw;  // (height, width) pairs, or the same numbers one after another
         items(a[1], levels, "level_hw must be a sequence of (height, width)", [&](Py_ssize_t, PyObject *l) {
             const auto put = [&](Py_ssize_t, PyObject *x) { hw.push_back(cut_integer32(x)); };
-            const bool row = PySequence_Check(l) && PySequence_Size(l) >= 0;
-            PyErr_Clear();  // (a number of an array type is a sequence without a length)
+            const bool row = PyObject_Size(l) >= 0;
+            PyErr_Clear();  // (a number has none)
             if (row) items(l, 2, "level_hw must be a sequence of (height, width)", put);
             else put(0, l);
         });
