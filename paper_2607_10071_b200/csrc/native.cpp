@@ -122,11 +122,16 @@ void tune(int32_t (&t)[4], PyObject *o)
     Py_DECREF(seq);
 }
 
-void *stream_of(PyObject *o, const at::Tensor &t)
-{
-    if (o == Py_None) return c10::cuda::getCurrentCUDAStream(t.get_device()).stream();
-    return reinterpret_cast<void *>(static_cast<uintptr_t>(integer(o)));
-}
+// The stream argument: None for the current one, or a cudaStream_t as an integer
+struct StreamArg {
+    bool current;
+    void *raw;
+    explicit StreamArg(PyObject *o)
+        : current(o == Py_None), raw(current ? nullptr : reinterpret_cast<void *>(static_cast<uintptr_t>(integer(o))))
+    {
+    }
+    void *on(const at::Tensor &t) const { return current ? c10::cuda::getCurrentCUDAStream(t.get_device()).stream() : raw; }
+};
 
 int32_t feature_dtype(const at::Tensor &t)
 {
@@ -138,6 +143,18 @@ int32_t feature_dtype(const at::Tensor &t)
 at::Tensor empty(std::initializer_list<int64_t> shape, at::ScalarType type, const at::Tensor &like)
 {
     return at::empty(shape, at::TensorOptions().dtype(type).device(like.device()));
+}
+
+// `body` without the interpreter lock: an allocation, a launch into a full queue or the memset of the backward may wait, and
+// the process's other Python threads go on meanwhile.  `body` touches no Python object.
+template <typename F>
+flashbev_status unlocked(F body)
+{
+    struct Unlock {
+        PyThreadState *state = PyEval_SaveThread();
+        ~Unlock() { PyEval_RestoreThread(state); }
+    } unlock;
+    return body();
 }
 
 PyObject *status(flashbev_status st) { return PyLong_FromLong(st); }
@@ -185,25 +202,25 @@ PyObject *py_sampling_vt(PyObject *, PyObject *const *a, Py_ssize_t n)
         items(a[4], 3, "grid must be (X, Y, Z)", [&](Py_ssize_t i, PyObject *v) { (i == 0 ? p.X : (i == 1 ? p.Y : p.Z)) = integer32(v); });
         p.reduce = integer32(a[5]), p.kernel = integer32(a[8]), p.out_dtype = integer32(a[12]);
         tune(p.tune, a[9]);
-        const c10::cuda::CUDAGuard guard(f.device());
-        at::Tensor out;
-        if (a[6] == Py_None) {
-            const auto type = p.out_dtype == FLASHBEV_F32 ? at::kFloat : at::kBFloat16;
-            out = nhwc ? empty({p.B, p.X, p.Y, p.C}, type, f) : empty({p.B, p.C, p.X, p.Y}, type, f);
-        } else {
-            out = tensor(a[6], "out");
-        }
-        p.features = f.data_ptr(), p.lidar2img = static_cast<const float *>(m.data_ptr()), p.out = out.data_ptr();
+        const StreamArg stream(a[10]);
+        at::Tensor out, scratch;
+        if (a[6] != Py_None) out = tensor(a[6], "out");
         if (a[7] != Py_None) p.valid_count_out = static_cast<int32_t *>(tensor(a[7], "valid_count").data_ptr());
-        at::Tensor scratch;
-        if (a[13] != Py_False && a[13] != Py_None) {
-            const size_t need = flashbev_workspace_bytes(&p);
+        const bool lend = a[13] != Py_False && a[13] != Py_None, own_scratch = a[13] == Py_True;
+        if (lend && !own_scratch && THPVariable_Check(a[13])) scratch = THPVariable_Unpack(a[13]);
+        const flashbev_status st = unlocked([&] {
+            const c10::cuda::CUDAGuard guard(f.device());
+            const auto type = p.out_dtype == FLASHBEV_F32 ? at::kFloat : at::kBFloat16;
+            if (!out.defined()) out = nhwc ? empty({p.B, p.X, p.Y, p.C}, type, f) : empty({p.B, p.C, p.X, p.Y}, type, f);
+            p.features = f.data_ptr(), p.lidar2img = static_cast<const float *>(m.data_ptr()), p.out = out.data_ptr();
+            const size_t need = lend ? flashbev_workspace_bytes(&p) : 0;
             if (need) {
-                scratch = a[13] == Py_True ? empty({(int64_t)need}, at::kByte, f) : tensor(a[13], "workspace");
+                if (own_scratch) scratch = empty({(int64_t)need}, at::kByte, f);
+                TORCH_CHECK_TYPE(scratch.defined(), "workspace must be True, False, None or a tensor");
                 p.workspace = scratch.data_ptr(), p.workspace_bytes = (size_t)scratch.numel() * scratch.element_size();
             }
-        }
-        const flashbev_status st = flashbev_sampling_vt(&p, stream_of(a[10], f));
+            return flashbev_sampling_vt(&p, stream.on(f));
+        });
         return st == FLASHBEV_OK ? THPVariable_Wrap(std::move(out)) : status(st);
     });
 }
@@ -233,11 +250,16 @@ PyObject *py_sampling_vt_backward(PyObject *, PyObject *const *a, Py_ssize_t n)
         Py_DECREF(z);
         p.reduce = integer32(a[6]);
         tune(p.tune, a[8]);
-        const c10::cuda::CUDAGuard guard(g.device());
-        at::Tensor out = a[7] == Py_None ? empty({p.B, p.N, p.feat_h, p.feat_w, p.C}, at::kFloat, g) : tensor(a[7], "grad_features");
-        p.grad_out = static_cast<const float *>(g.data_ptr()), p.lidar2img = static_cast<const float *>(m.data_ptr());
-        p.grad_features = static_cast<float *>(out.data_ptr());
-        const flashbev_status st = flashbev_sampling_vt_backward(&p, stream_of(a[9], g));
+        const StreamArg stream(a[9]);
+        at::Tensor out;
+        if (a[7] != Py_None) out = tensor(a[7], "grad_features");
+        const flashbev_status st = unlocked([&] {
+            const c10::cuda::CUDAGuard guard(g.device());
+            if (!out.defined()) out = empty({p.B, p.N, p.feat_h, p.feat_w, p.C}, at::kFloat, g);
+            p.grad_out = static_cast<const float *>(g.data_ptr()), p.lidar2img = static_cast<const float *>(m.data_ptr());
+            p.grad_features = static_cast<float *>(out.data_ptr());
+            return flashbev_sampling_vt_backward(&p, stream.on(g));
+        });
         return st == FLASHBEV_OK ? THPVariable_Wrap(std::move(out)) : status(st);
     });
 }
@@ -267,31 +289,33 @@ PyObject *py_sampling_vt_multires(PyObject *, PyObject *const *a, Py_ssize_t n)
         items(a[4], 3, "grid must be (X, Y, Z)", [&](Py_ssize_t i, PyObject *v) { (i == 0 ? p.X : (i == 1 ? p.Y : p.Z)) = integer32(v); });
         p.reduce = integer32(a[5]), p.kernel = integer32(a[8]), p.out_dtype = FLASHBEV_F32;
         tune(p.tune, a[9]);
-        const c10::cuda::CUDAGuard guard(f0.device());
-        at::Tensor out;
-        if (a[6] == Py_None) out = nhwc ? empty({p.B, p.X, p.Y, p.C}, at::kFloat, f0) : empty({p.B, p.C, p.X, p.Y}, at::kFloat, f0);
-        else out = tensor(a[6], "out");
-        p.lidar2img = static_cast<const float *>(m.data_ptr()), p.out = out.data_ptr();
+        const StreamArg stream(a[10]);
+        at::Tensor out, scratch;
+        if (a[6] != Py_None) out = tensor(a[6], "out");
         if (a[7] != Py_None) p.valid_count_out = static_cast<int32_t *>(tensor(a[7], "valid_count").data_ptr());
-        // planar tensors and ragged channel counts: lend the scratch of the largest level (the levels run one after another)
-        std::vector<const void *> ptrs;
-        std::vector<int32_t> hw;
-        size_t need = 0;
-        for (const at::Tensor &f : maps) {
-            ptrs.push_back(f.data_ptr());
-            hw.push_back((int32_t)f.size(nhwc ? 2 : 3)), hw.push_back((int32_t)f.size(nhwc ? 3 : 4));
-            p.features = ptrs.back(), p.feat_h = hw[hw.size() - 2], p.feat_w = hw.back();
-            need = std::max(need, flashbev_workspace_bytes(&p));
-        }
-        p.features = ptrs[0], p.feat_h = hw[0], p.feat_w = hw[1];
-        at::Tensor scratch;
-        if (need) {
-            scratch = empty({(int64_t)need}, at::kByte, f0);
-            p.workspace = scratch.data_ptr(), p.workspace_bytes = need;
-        }
-        flashbev_vt_multires_params q = {};
-        q.struct_size = sizeof(q), q.base = &p, q.levels = (int32_t)levels, q.features = ptrs.data(), q.feat_hw = hw.data();
-        const flashbev_status st = flashbev_sampling_vt_multires(&q, stream_of(a[10], f0));
+        const flashbev_status st = unlocked([&] {
+            const c10::cuda::CUDAGuard guard(f0.device());
+            if (!out.defined()) out = nhwc ? empty({p.B, p.X, p.Y, p.C}, at::kFloat, f0) : empty({p.B, p.C, p.X, p.Y}, at::kFloat, f0);
+            p.lidar2img = static_cast<const float *>(m.data_ptr()), p.out = out.data_ptr();
+            // planar tensors and ragged channel counts: lend the scratch of the largest level (the levels run one after another)
+            std::vector<const void *> ptrs;
+            std::vector<int32_t> hw;
+            size_t need = 0;
+            for (const at::Tensor &f : maps) {
+                ptrs.push_back(f.data_ptr());
+                hw.push_back((int32_t)f.size(nhwc ? 2 : 3)), hw.push_back((int32_t)f.size(nhwc ? 3 : 4));
+                p.features = ptrs.back(), p.feat_h = hw[hw.size() - 2], p.feat_w = hw.back();
+                need = std::max(need, flashbev_workspace_bytes(&p));
+            }
+            p.features = ptrs[0], p.feat_h = hw[0], p.feat_w = hw[1];
+            if (need) {
+                scratch = empty({(int64_t)need}, at::kByte, f0);
+                p.workspace = scratch.data_ptr(), p.workspace_bytes = need;
+            }
+            flashbev_vt_multires_params q = {};
+            q.struct_size = sizeof(q), q.base = &p, q.levels = (int32_t)levels, q.features = ptrs.data(), q.feat_hw = hw.data();
+            return flashbev_sampling_vt_multires(&q, stream.on(f0));
+        });
         return st == FLASHBEV_OK ? THPVariable_Wrap(std::move(out)) : status(st);
     });
 }
@@ -325,14 +349,19 @@ PyObject *py_sca(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (hw.size() < 2 * (size_t)p.L) value_error("level_hw must have an entry per level");
         geometry(p, a[5], a[6]);
         items(a[7], 3, "grid must be (X, Y, Zref)", [&](Py_ssize_t i, PyObject *x) { (i == 0 ? p.X : (i == 1 ? p.Y : p.Zref)) = integer32(x); });
-        const c10::cuda::CUDAGuard guard(v.device());
-        at::Tensor out = a[8] == Py_None ? empty({p.B, (int64_t)p.X * p.Y, (int64_t)p.heads * p.head_dim}, at::kFloat, v) : tensor(a[8], "out");
-        p.value = v.data_ptr(), p.level_hw = hw.data(), p.lidar2img = static_cast<const float *>(m.data_ptr());
-        p.offsets = static_cast<const float *>(o.data_ptr()), p.weights = static_cast<const float *>(w.data_ptr());
-        p.out = static_cast<float *>(out.data_ptr());
-        if (a[9] != Py_None) p.hits_out = static_cast<int32_t *>(tensor(a[9], "hits").data_ptr());
         p.chunk_records = cut_integer32(a[11]);
-        const flashbev_status st = flashbev_sca(&p, stream_of(a[10], v));
+        const StreamArg stream(a[10]);
+        at::Tensor out;
+        if (a[8] != Py_None) out = tensor(a[8], "out");
+        if (a[9] != Py_None) p.hits_out = static_cast<int32_t *>(tensor(a[9], "hits").data_ptr());
+        const flashbev_status st = unlocked([&] {
+            const c10::cuda::CUDAGuard guard(v.device());
+            if (!out.defined()) out = empty({p.B, (int64_t)p.X * p.Y, (int64_t)p.heads * p.head_dim}, at::kFloat, v);
+            p.value = v.data_ptr(), p.level_hw = hw.data(), p.lidar2img = static_cast<const float *>(m.data_ptr());
+            p.offsets = static_cast<const float *>(o.data_ptr()), p.weights = static_cast<const float *>(w.data_ptr());
+            p.out = static_cast<float *>(out.data_ptr());
+            return flashbev_sca(&p, stream.on(v));
+        });
         return st == FLASHBEV_OK ? THPVariable_Wrap(std::move(out)) : status(st);
     });
 }

@@ -68,3 +68,44 @@ def test_failed_allocation_is_an_out_of_memory_error_and_leaves_the_device_usabl
     out = fb.sampling_vt(f, m, *geo, (4, 4, 1))
     torch.cuda.synchronize()
     assert out.shape == (1, 4, 4, 512) and bool(torch.isfinite(out).all())
+
+
+@pytest.mark.gpu
+def test_other_threads_run_while_a_call_waits():
+    """A call that finds the stream's launch queue full waits for room in it, without the interpreter lock."""
+    import threading
+    import time
+
+    import torch
+    dev = torch.device("cuda:0")
+    f, m = torch.ones((1, 2, 4, 6, 8), device=dev), torch.eye(4, device=dev).expand(1, 2, 4, 4).contiguous()
+    out = torch.empty((1, 4, 4, 8), device=dev)
+    fb.sampling_vt(f, m, (32, 48), RANGE, (4, 4, 1), out=out)
+    torch.cuda.synchronize()
+    ticks, stop = [], threading.Event()
+
+    def tick():
+        while not stop.is_set():
+            ticks.append(time.perf_counter())
+            time.sleep(0.001)
+
+    thread = threading.Thread(target=tick)
+    thread.start()
+    try:
+        torch.cuda._sleep(1_000_000_000)           # half a second of an idle GPU at the head of the stream
+        longest = (0.0, 0.0)
+        for _ in range(20000):
+            t0 = time.perf_counter()
+            fb.sampling_vt(f, m, (32, 48), RANGE, (4, 4, 1), out=out)
+            longest = max(longest, (time.perf_counter() - t0, t0))
+            if longest[0] > 0.1:
+                break
+        torch.cuda.synchronize()
+    finally:
+        stop.set()
+        thread.join()
+    waited, since = longest
+    assert waited > 0.1, "no call had to wait"
+    during = [t for t in ticks if since < t < since + waited]
+    gaps = [b - a for a, b in zip([since] + during, during + [since + waited])]
+    assert max(gaps) < 0.5 * waited, f"the other thread stood still for {max(gaps):.3f} s of a wait of {waited:.3f} s"
