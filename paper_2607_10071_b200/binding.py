@@ -340,7 +340,8 @@ def sampling_vt(features, lidar2img, img_hw, bev_range, grid, reduce=REDUCE_SUM,
     [B,C,X,Y] (NCHW), float32 or bfloat16 per ``out_dtype`` (allocated by torch if ``out`` is None).
     ``workspace``: for NCHW tensors and for channel counts that are not whole 16-byte vectors, lend the call the
     scratch ``flashbev_workspace_bytes`` asks for (a torch allocation, or a uint8 CUDA tensor of the caller's);
-    False: none, the generic kernel runs."""
+    False: none, the generic kernel runs.  ``stream``: a raw cudaStream_t instead of the current stream; scratch and a new
+    result are allocated for it, and the caller orders the streams."""
     return _result((_native or native()).sampling_vt(features, lidar2img, img_hw, bev_range, grid, reduce, out, valid_count,
                                                      kernel, tune, stream, layout, out_dtype, workspace), "flashbev_sampling_vt")
 

@@ -130,7 +130,37 @@ struct StreamArg {
         : current(o == Py_None), raw(current ? nullptr : reinterpret_cast<void *>(static_cast<uintptr_t>(integer(o))))
     {
     }
-    void *on(const at::Tensor &t) const { return current ? c10::cuda::getCurrentCUDAStream(t.get_device()).stream() : raw; }
+};
+
+// A call's device and stream.  A stream that the caller names is the current one while this object lives, so that the allocator
+// hands out memory that belongs to it: scratch is free again when the call returns, and only later work of the same stream may
+// get it, and what an earlier owner still does on another stream is not written over.  (Memory of the current stream, written
+// on another one, was open to both.)
+class Place {
+    const c10::cuda::CUDAGuard device_;
+    c10::cuda::OptionalCUDAStreamGuard named_;
+    void *stream_;
+    c10::cuda::CUDAStream caller_;
+
+public:
+    Place(const at::Tensor &t, const StreamArg &s)
+        : device_(t.device()), stream_(s.raw), caller_(c10::cuda::getCurrentCUDAStream(t.get_device()))
+    {
+        if (s.current) stream_ = caller_.stream();
+        if (stream_ == caller_.stream()) return;
+        // (the legacy stream has a handle of its own beside NULL)
+        const cudaStream_t raw = static_cast<cudaStream_t>(stream_);
+        named_.reset_stream(raw == cudaStreamLegacy ? c10::cuda::getDefaultCUDAStream(t.get_device())
+                                                    : c10::cuda::getStreamFromExternal(raw, t.get_device()));
+    }
+    void *stream() const { return stream_; }
+
+    // A result: the caller goes on with it on the stream that was current, and drops it at any time.
+    at::Tensor result(at::Tensor t) const
+    {
+        if (stream_ != caller_.stream()) t.record_stream(caller_.unwrap());
+        return t;
+    }
 };
 
 int32_t feature_dtype(const at::Tensor &t)
@@ -209,9 +239,10 @@ PyObject *py_sampling_vt(PyObject *, PyObject *const *a, Py_ssize_t n)
         const bool lend = a[13] != Py_False && a[13] != Py_None, own_scratch = a[13] == Py_True;
         if (lend && !own_scratch && THPVariable_Check(a[13])) scratch = THPVariable_Unpack(a[13]);
         const flashbev_status st = unlocked([&] {
-            const c10::cuda::CUDAGuard guard(f.device());
+            const Place place(f, stream);
             const auto type = p.out_dtype == FLASHBEV_F32 ? at::kFloat : at::kBFloat16;
-            if (!out.defined()) out = nhwc ? empty({p.B, p.X, p.Y, p.C}, type, f) : empty({p.B, p.C, p.X, p.Y}, type, f);
+            if (!out.defined())
+                out = place.result(nhwc ? empty({p.B, p.X, p.Y, p.C}, type, f) : empty({p.B, p.C, p.X, p.Y}, type, f));
             p.features = f.data_ptr(), p.lidar2img = static_cast<const float *>(m.data_ptr()), p.out = out.data_ptr();
             const size_t need = lend ? flashbev_workspace_bytes(&p) : 0;
             if (need) {
@@ -219,7 +250,7 @@ PyObject *py_sampling_vt(PyObject *, PyObject *const *a, Py_ssize_t n)
                 TORCH_CHECK_TYPE(scratch.defined(), "workspace must be True, False, None or a tensor");
                 p.workspace = scratch.data_ptr(), p.workspace_bytes = (size_t)scratch.numel() * scratch.element_size();
             }
-            return flashbev_sampling_vt(&p, stream.on(f));
+            return flashbev_sampling_vt(&p, place.stream());
         });
         return st == FLASHBEV_OK ? THPVariable_Wrap(std::move(out)) : status(st);
     });
@@ -254,11 +285,11 @@ PyObject *py_sampling_vt_backward(PyObject *, PyObject *const *a, Py_ssize_t n)
         at::Tensor out;
         if (a[7] != Py_None) out = tensor(a[7], "grad_features");
         const flashbev_status st = unlocked([&] {
-            const c10::cuda::CUDAGuard guard(g.device());
-            if (!out.defined()) out = empty({p.B, p.N, p.feat_h, p.feat_w, p.C}, at::kFloat, g);
+            const Place place(g, stream);
+            if (!out.defined()) out = place.result(empty({p.B, p.N, p.feat_h, p.feat_w, p.C}, at::kFloat, g));
             p.grad_out = static_cast<const float *>(g.data_ptr()), p.lidar2img = static_cast<const float *>(m.data_ptr());
             p.grad_features = static_cast<float *>(out.data_ptr());
-            return flashbev_sampling_vt_backward(&p, stream.on(g));
+            return flashbev_sampling_vt_backward(&p, place.stream());
         });
         return st == FLASHBEV_OK ? THPVariable_Wrap(std::move(out)) : status(st);
     });
@@ -294,8 +325,9 @@ PyObject *py_sampling_vt_multires(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (a[6] != Py_None) out = tensor(a[6], "out");
         if (a[7] != Py_None) p.valid_count_out = static_cast<int32_t *>(tensor(a[7], "valid_count").data_ptr());
         const flashbev_status st = unlocked([&] {
-            const c10::cuda::CUDAGuard guard(f0.device());
-            if (!out.defined()) out = nhwc ? empty({p.B, p.X, p.Y, p.C}, at::kFloat, f0) : empty({p.B, p.C, p.X, p.Y}, at::kFloat, f0);
+            const Place place(f0, stream);
+            if (!out.defined())
+                out = place.result(nhwc ? empty({p.B, p.X, p.Y, p.C}, at::kFloat, f0) : empty({p.B, p.C, p.X, p.Y}, at::kFloat, f0));
             p.lidar2img = static_cast<const float *>(m.data_ptr()), p.out = out.data_ptr();
             // planar tensors and ragged channel counts: lend the scratch of the largest level (the levels run one after another)
             std::vector<const void *> ptrs;
@@ -314,7 +346,7 @@ PyObject *py_sampling_vt_multires(PyObject *, PyObject *const *a, Py_ssize_t n)
             }
             flashbev_vt_multires_params q = {};
             q.struct_size = sizeof(q), q.base = &p, q.levels = (int32_t)levels, q.features = ptrs.data(), q.feat_hw = hw.data();
-            return flashbev_sampling_vt_multires(&q, stream.on(f0));
+            return flashbev_sampling_vt_multires(&q, place.stream());
         });
         return st == FLASHBEV_OK ? THPVariable_Wrap(std::move(out)) : status(st);
     });
@@ -355,12 +387,12 @@ PyObject *py_sca(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (a[8] != Py_None) out = tensor(a[8], "out");
         if (a[9] != Py_None) p.hits_out = static_cast<int32_t *>(tensor(a[9], "hits").data_ptr());
         const flashbev_status st = unlocked([&] {
-            const c10::cuda::CUDAGuard guard(v.device());
-            if (!out.defined()) out = empty({p.B, (int64_t)p.X * p.Y, (int64_t)p.heads * p.head_dim}, at::kFloat, v);
+            const Place place(v, stream);
+            if (!out.defined()) out = place.result(empty({p.B, (int64_t)p.X * p.Y, (int64_t)p.heads * p.head_dim}, at::kFloat, v));
             p.value = v.data_ptr(), p.level_hw = hw.data(), p.lidar2img = static_cast<const float *>(m.data_ptr());
             p.offsets = static_cast<const float *>(o.data_ptr()), p.weights = static_cast<const float *>(w.data_ptr());
             p.out = static_cast<float *>(out.data_ptr());
-            return flashbev_sca(&p, stream.on(v));
+            return flashbev_sca(&p, place.stream());
         });
         return st == FLASHBEV_OK ? THPVariable_Wrap(std::move(out)) : status(st);
     });

@@ -109,3 +109,65 @@ def test_other_threads_run_while_a_call_waits():
     during = [t for t in ticks if since < t < since + waited]
     gaps = [b - a for a, b in zip([since] + during, during + [since + waited])]
     assert max(gaps) < 0.5 * waited, f"the other thread stood still for {max(gaps):.3f} s of a wait of {waited:.3f} s"
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("call", ["planar", "ragged", "pyramid"])
+def test_memory_of_a_call_on_a_named_stream_belongs_to_that_stream(call):
+    """Scratch and result come from the named stream's memory: what is allocated later for another stream never gets the scratch
+    while the call may still use it, and a dropped result is not handed out again while the caller's stream may still read it."""
+    import torch
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(5)
+    m = torch.eye(4, device=dev).expand(1, 2, 4, 4).contiguous()
+    m[:, :, :3, 3] = torch.tensor([24.0, 16.0, 4.0], device=dev)
+    img, r, grid = (32, 48), (-1.0, 1.0, -1.0, 1.0, -1.0, 1.0), (90, 90, 4)
+    C = 30 if call == "ragged" else 32
+    shape = (1, 2, 120, 170, C) if call == "ragged" else (1, 2, C, 120, 170)
+    f = torch.randn(shape, generator=gen, device=dev)
+    layout = fb.NHWC if call == "ragged" else fb.NCHW
+
+    def run(**kw):
+        if call == "pyramid":
+            return fb.sampling_vt_multires([f, f], m, img, r, grid, layout=layout, **kw)
+        return fb.sampling_vt(f, m, img, r, grid, layout=layout, **kw)
+
+    want = run()
+    assert fb.flashbev_last_kernel_name().startswith("tiled")
+    side = torch.cuda.Stream()
+    out = torch.empty_like(want)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    before = {s["address"] for s in torch.cuda.memory_snapshot()}
+    run(out=out, stream=side.cuda_stream)
+    fresh = [s for s in torch.cuda.memory_snapshot() if s["address"] not in before]
+    scratch = 2 * 120 * 170 * 32 * 4
+    assert sum(s["total_size"] for s in fresh) >= scratch, "the scratch was not allocated in this call"
+    assert {s["stream"] for s in fresh} == {side.cuda_stream}
+    side.synchronize()
+    assert torch.equal(out, want)
+    # a result of the call: the named stream's memory, kept while the caller's stream still works with it
+    res = run(stream=side.cuda_stream)
+    where = res.data_ptr()
+    assert any(s["address"] <= where < s["address"] + s["total_size"] for s in torch.cuda.memory_snapshot()
+               if s["stream"] == side.cuda_stream)
+    torch.cuda.current_stream().wait_stream(side)
+    torch.cuda._sleep(200_000_000)
+    copy = res.clone()
+    del res
+    again = run(stream=side.cuda_stream)
+    assert again.data_ptr() != where
+    torch.cuda.synchronize()
+    assert torch.equal(copy, want) and torch.equal(again, want)
+
+
+@pytest.mark.gpu
+def test_default_stream_handles():
+    import torch
+    dev = torch.device("cuda:0")
+    f, m = torch.ones((1, 2, 4, 6, 8), device=dev), torch.eye(4, device=dev).expand(1, 2, 4, 4).contiguous()
+    want = fb.sampling_vt(f, m, (32, 48), RANGE, (4, 4, 1))
+    for handle in (0, 1, 2):                       # NULL, the legacy stream's and the per-thread stream's own handles
+        got = fb.sampling_vt(f, m, (32, 48), RANGE, (4, 4, 1), stream=handle)
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
