@@ -4,6 +4,7 @@ from __future__ import annotations
 import importlib.util
 import os
 import subprocess
+import sys
 import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -30,8 +31,23 @@ def needs_build(lib: str = LIB) -> bool:
     return any(os.path.getmtime(s) > t for s in SOURCES + HEADERS)
 
 
+def native_prerequisites() -> str | None:
+    """What the extension module needs and this machine lacks (None: nothing).  The library itself needs none of it."""
+    spec = importlib.util.find_spec("torch")
+    if spec is None or not spec.submodule_search_locations:
+        return "PyTorch is not installed"
+    if not os.path.exists(os.path.join(spec.submodule_search_locations[0], "lib", "libc10_cuda.so")):
+        return "the installed PyTorch has no CUDA part"
+    if not os.path.exists(os.path.join(sysconfig.get_paths()["include"], "Python.h")):
+        return "the headers of Python are not installed"
+    return None
+
+
 def build_native(force: bool = False) -> str:
     """Compile csrc/native.cpp (g++, PyTorch headers) into the extension module next to this file; returns its path."""
+    missing = native_prerequisites()
+    if missing:
+        raise RuntimeError(f"the extension module for torch tensors cannot be built: {missing}")
     sources = NATIVE_SOURCES + HEADERS[:1]
     if force or not os.path.exists(NATIVE) or any(os.path.getmtime(s) > os.path.getmtime(NATIVE) for s in sources):
         torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
@@ -46,7 +62,8 @@ def build_native(force: bool = False) -> str:
 
 
 def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False) -> str:
-    """Compile csrc/*.cu into libflashbev.so next to this file (and the extension module over it); returns its path.
+    """Compile csrc/*.cu into libflashbev.so next to this file, and the extension module over it where PyTorch is installed;
+    returns the library's path.
 
     ``debug_bounds``: build libflashbev_debug_bounds.so instead, with -DFLASHBEV_DEBUG_BOUNDS: every index the
     tiled kernel computes is range-checked, violations are counted into the caller's ``debug_error_word`` and
@@ -58,7 +75,11 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
                (["-Xptxas", "-v"] if verbose else []) + SOURCES + ["-o", lib])
         subprocess.run(cmd, check=True)
     if not debug_bounds:
-        build_native(force)
+        missing = native_prerequisites()
+        if missing:  # the C ABI and its ctypes mirror work without; calls with torch tensors raise ImportError
+            print(f"libflashbev.so only, no extension module for torch tensors: {missing}", file=sys.stderr)
+        else:
+            build_native(force)
     return lib
 
 
