@@ -1,6 +1,7 @@
 """Build the CUDA library in-tree for sm_100a (nvcc cross-compiles without a GPU) and its CPython entry points."""
 from __future__ import annotations
 
+import importlib.metadata
 import importlib.util
 import os
 import subprocess
@@ -22,6 +23,7 @@ LIB_DEBUG_BOUNDS = os.path.join(_HERE, "libflashbev_debug_bounds.so")
 
 NATIVE_SOURCES = [os.path.join(_HERE, "csrc", "native.cpp")]
 NATIVE = os.path.join(_HERE, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
+NATIVE_RECORD = os.path.join(_HERE, "_native.built_with")  # what NATIVE was built with
 
 
 def needs_build(lib: str = LIB) -> bool:
@@ -43,13 +45,27 @@ def native_prerequisites() -> str | None:
     return None
 
 
+def _built_with() -> str:
+    """What the extension module is bound to beside its sources: it calls PyTorch's C++ libraries, whose classes and symbols
+    change from version to version."""
+    return f"torch {importlib.metadata.version('torch')}\n"
+
+
+def needs_native_build() -> bool:
+    if not os.path.exists(NATIVE) or not os.path.exists(NATIVE_RECORD):
+        return True
+    with open(NATIVE_RECORD) as f:
+        if f.read() != _built_with():
+            return True
+    return any(os.path.getmtime(s) > os.path.getmtime(NATIVE) for s in NATIVE_SOURCES + HEADERS[:1])
+
+
 def build_native(force: bool = False) -> str:
     """Compile csrc/native.cpp (g++, PyTorch headers) into the extension module next to this file; returns its path."""
     missing = native_prerequisites()
     if missing:
         raise RuntimeError(f"the extension module for torch tensors cannot be built: {missing}")
-    sources = NATIVE_SOURCES + HEADERS[:1]
-    if force or not os.path.exists(NATIVE) or any(os.path.getmtime(s) > os.path.getmtime(NATIVE) for s in sources):
+    if force or needs_native_build():
         torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
         inc = [os.path.join(torch_dir, "include"), os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"),
                sysconfig.get_paths()["include"], "/usr/local/cuda/include", os.path.join(ROOT, "include")]
@@ -58,6 +74,8 @@ def build_native(force: bool = False) -> str:
                [f"-L{os.path.join(torch_dir, 'lib')}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda",
                 f"-L{_HERE}", "-lflashbev", "-Wl,-rpath,$ORIGIN", "-o", NATIVE])
         subprocess.run(cmd, check=True)
+        with open(NATIVE_RECORD, "w") as f:
+            f.write(_built_with())
     return NATIVE
 
 

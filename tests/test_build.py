@@ -1,4 +1,5 @@
 """The build rules, with the compilers replaced by a recorder."""
+import importlib.metadata
 import importlib.util
 import os
 
@@ -17,7 +18,7 @@ def compiled(monkeypatch, tmp_path):
         done.append(os.path.basename(out))
         open(out, "w").close()
 
-    for name in ("LIB", "LIB_DEBUG_BOUNDS", "NATIVE"):
+    for name in ("LIB", "LIB_DEBUG_BOUNDS", "NATIVE", "NATIVE_RECORD"):
         monkeypatch.setattr(fbuild, name, str(tmp_path / os.path.basename(getattr(fbuild, name))))
     monkeypatch.setattr(fbuild.subprocess, "run", run)
     return done
@@ -44,3 +45,20 @@ def test_library_and_extension_build_with_pytorch(compiled):
     assert compiled == ["libflashbev.so", os.path.basename(fbuild.NATIVE)]
     fbuild.build()                                 # up to date
     assert len(compiled) == 2
+
+
+def test_extension_is_rebuilt_for_another_pytorch(compiled, monkeypatch):
+    if fbuild.native_prerequisites():
+        pytest.skip(fbuild.native_prerequisites())
+    name = os.path.basename(fbuild.NATIVE)
+    fbuild.build_native()
+    fbuild.build_native()
+    assert compiled == [name]
+    version = importlib.metadata.version
+    monkeypatch.setattr(importlib.metadata, "version", lambda p: "99.0" if p == "torch" else version(p))
+    fbuild.build_native()
+    fbuild.build_native()
+    assert compiled == [name, name]
+    os.remove(fbuild.NATIVE_RECORD)                # built by hand, or by an older rule: nothing says what with
+    fbuild.build_native()
+    assert compiled == [name, name, name]
