@@ -429,11 +429,14 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // EVEN: every lane has a head in every pass (heads = V * heads per pass, 32 lanes all used)
-// bf16 takes seven CTAs per SM (72 registers): the gather waits on L2 most of the time.  N = 6, C = 256, 200 x 200, P = 8:
-// 309 / 282 / 274 / 378 us at 5 / 6 / 7 / 8.  fp32 moves twice the bytes through L1 and gains nothing (363 / 362 / 364 us),
-// a 120 x 90 grid loses 3 %: five.
+// bf16 with one head per lane (V = 1, 70 registers) takes seven CTAs per SM: the gather waits on L2 most of the time.  N = 6,
+// L = 4, P = 8, 5 / 6 / 7 CTAs: 8 heads of 32, 200 x 200 309 / 282 / 270 us, 120 x 90 105 / 97 / 94, 50 x 50 45.3 / 45.3 / 46.0; 6 of
+// 32, 200 x 200 327 / 302 / 282; 2 of 128 243 / 220 / 208.  With two heads per lane 72 registers do not hold the loop (uneven
+// heads: 116 bytes of spill stores, 240 of loads): 16 of 32, 200 x 200 546 / 544 / 551 us, 50 x 50 81 / 88 / 110; 12 of 32 517 /
+// 570 / 613 and 68 / 80 / 90; 8 of 64 443 / 429 / 445 and 69 / 75 / 99: five.  fp32 moves twice the bytes through L1 and gains
+// nothing (8 of 32: 363 / 362 / 364 us), a 120 x 90 grid loses 3 %: five.
 template <int V, bool EVEN, bool BF16>
-__global__ void __launch_bounds__(128, V <= 2 ? (BF16 ? 7 : 5) : 3) sca_kernel(const ScaParams p)
+__global__ void __launch_bounds__(128, V == 1 && BF16 ? 7 : (V <= 2 ? 5 : 3)) sca_kernel(const ScaParams p)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr unsigned FULL = 0xffffffffu;

@@ -72,6 +72,14 @@ def test_bf16_values(oracle, general, heads, Dh):
     check(oracle, c, f"bf16 heads={heads} Dh={Dh}", bf16=True)
 
 
+@pytest.mark.parametrize("heads,Dh", [(16, 32), (12, 32), (8, 64), (9, 32), (64, 8), (3, 128)])
+def test_bf16_two_heads_per_lane(oracle, heads, Dh):
+    """Even and uneven distributions of the heads over a warp that has to take them in two passes."""
+    c = make_case(heads * 100 + Dh + 11, B=1, N=6, heads=heads, Dh=Dh, levels=((12, 18), (6, 9)), P=4,
+                  grid=(9, 7, 2), general=True, rng_xy=10.0)
+    check(oracle, c, f"bf16 heads={heads} Dh={Dh}", bf16=True)
+
+
 def test_bf16_unsupported_shapes():
     import torch
     c = make_case(5, N=2, heads=2, Dh=4, grid=(4, 4, 2))
