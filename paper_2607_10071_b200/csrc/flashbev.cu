@@ -869,10 +869,11 @@ int padded_channels(const flashbev_vt_params *p)
     return (p->C + vec - 1) / vec * vec;
 }
 
-// Bytes of the channels-last copy of NCHW features (0: not worth it, or the shape cannot take the tiled kernel).  Channel
-// counts that are not whole vectors are padded in the copy.  Grids of fewer than 12 K bins keep the generic kernel for those (one
-// launch, no scratch to find for callers of the smallest grids; 30-45 us either way of the line).  Measured with six 29 x 77
-// maps of 97 bf16 channels: 53 -> 20 us on 64 x 64 x 8 bins, 485 -> 62 us on 200 x 200 x 16.
+// Bytes of the channels-last copy of NCHW features (0: the call takes no scratch).  Channel counts that are not whole vectors are
+// padded in the copy, from 12288 bins on.  Smaller grids ask for no scratch and run in one launch of the generic kernel: that is
+// the contract of flashbev_workspace_bytes, kept for the callers that rely on it and not for speed.  The copy and the tiled kernel win on both sides of the
+// line (N = 6, generic / tiled): 97 bf16 channels of 29 x 77, 50 x 50 x 4 bins 37.7 / 14.8 us, 64 x 48 x 4 33.7 / 14.8, 64 x 64 x 8
+// 50.9 / 18.1; 30 fp32 of 16 x 44, 34.7 / 9.3, 31.7 / 9.2, 41.2 / 10.2; 82 fp32 of 32 x 88, 44.6 / 16.8, 35.2 / 17.1, 59.3 / 23.9.
 size_t nchw_copy_bytes(const flashbev_vt_params *p)
 {
     if (p->layout != FLASHBEV_NCHW) return 0;
