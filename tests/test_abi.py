@@ -133,12 +133,10 @@ def test_workspace_is_asked_for_planar_tensors_only():
 
 
 def test_workspace_of_planar_tensors_with_ragged_channel_counts_starts_at_its_stated_line():
-    bins = {(64, 48, 4): True, (63, 65, 3): False, (4095, 1, 3): False, (4096, 1, 3): True}
-    for (X, Y, Z), asked in bins.items():
-        p = good_params(layout=fb.NCHW, C=30, X=X, Y=Y, Z=Z)
-        assert (fb.flashbev_workspace_bytes(p) > 0) == asked, (X, Y, Z)
-        assert fb.flashbev_workspace_bytes(good_params(layout=fb.NCHW, C=32, X=X, Y=Y, Z=Z)) > 0
-        assert fb.flashbev_workspace_bytes(good_params(C=30, X=X, Y=Y, Z=Z)) > 0
+    for grid, asked in (((64, 48, 4), True), ((63, 65, 3), False), ((4095, 1, 3), False), ((4096, 1, 3), True)):
+        assert (fb.flashbev_workspace_bytes(good_params(layout=fb.NCHW, C=30, grid=grid)) > 0) == asked, grid
+        assert fb.flashbev_workspace_bytes(good_params(layout=fb.NCHW, C=32, grid=grid)) > 0
+        assert fb.flashbev_workspace_bytes(good_params(C=30, grid=grid)) > 0
 
 
 def test_multires_arguments_are_validated_on_the_host():
