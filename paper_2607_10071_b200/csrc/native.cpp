@@ -229,7 +229,8 @@ PyObject *py_sampling_vt(PyObject *, PyObject *const *a, Py_ssize_t n)
         p.B = (int32_t)f.size(0), p.N = (int32_t)f.size(1), p.C = (int32_t)f.size(nhwc ? 4 : 2);
         p.feat_h = (int32_t)f.size(nhwc ? 2 : 3), p.feat_w = (int32_t)f.size(nhwc ? 3 : 4);
         geometry(p, a[2], a[3]);
-        items(a[4], 3, "grid must be (X, Y, Z)", [&](Py_ssize_t i, PyObject *v) { (i == 0 ? p.X : (i == 1 ? p.Y : p.Z)) = integer32(v); });
+        int32_t *const axis[3] = {&p.X, &p.Y, &p.Z};
+        items(a[4], 3, "grid must be (X, Y, Z)", [&](Py_ssize_t i, PyObject *v) { *axis[i] = integer32(v); });
         p.reduce = integer32(a[5]), p.kernel = integer32(a[8]), p.out_dtype = integer32(a[12]);
         tune(p.tune, a[9]);
         const StreamArg stream(a[10]);
@@ -262,7 +263,8 @@ PyObject *py_sampling_vt_backward(PyObject *, PyObject *const *a, Py_ssize_t n)
     return guarded([&]() -> PyObject * {
         need_args(n, 10);
         const at::Tensor &g = tensor(a[0], "grad_out"), &m = tensor(a[1], "lidar2img");
-        if (!g.is_cuda() || g.scalar_type() != at::kFloat || !g.is_contiguous()) value_error("grad_out must be a contiguous CUDA float32 tensor");
+        if (!g.is_cuda() || g.scalar_type() != at::kFloat || !g.is_contiguous())
+            value_error("grad_out must be a contiguous CUDA float32 tensor");
         if (g.dim() != 4) value_error("grad_out must have four dimensions");
         flashbev_vt_backward_params p = {};
         p.struct_size = sizeof(p);
@@ -304,7 +306,8 @@ PyObject *py_sampling_vt_multires(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (levels < 0) throw Bad();
         if (levels < 1) value_error("at least one level is needed");
         std::vector<at::Tensor> maps;
-        items(a[0], levels, "features must be a sequence of tensors", [&](Py_ssize_t, PyObject *v) { maps.push_back(tensor(v, "features")); });
+        items(a[0], levels, "features must be a sequence of tensors",
+              [&](Py_ssize_t, PyObject *v) { maps.push_back(tensor(v, "features")); });
         const at::Tensor &f0 = maps[0], &m = tensor(a[1], "lidar2img");
         for (const at::Tensor &f : maps)
             if (!f.is_cuda() || !f.is_contiguous() || f.dtype() != f0.dtype() || f.dim() != 5)
@@ -312,12 +315,14 @@ PyObject *py_sampling_vt_multires(PyObject *, PyObject *const *a, Py_ssize_t n)
         flashbev_vt_params p = {};
         p.struct_size = sizeof(p);
         p.feat_dtype = feature_dtype(f0);
-        if (!m.is_cuda() || m.scalar_type() != at::kFloat || !m.is_contiguous()) value_error("lidar2img must be a contiguous CUDA float32 tensor");
+        if (!m.is_cuda() || m.scalar_type() != at::kFloat || !m.is_contiguous())
+            value_error("lidar2img must be a contiguous CUDA float32 tensor");
         p.layout = integer32(a[11]);
         const bool nhwc = p.layout == FLASHBEV_NHWC;
         p.B = (int32_t)f0.size(0), p.N = (int32_t)f0.size(1), p.C = (int32_t)f0.size(nhwc ? 4 : 2);
         geometry(p, a[2], a[3]);
-        items(a[4], 3, "grid must be (X, Y, Z)", [&](Py_ssize_t i, PyObject *v) { (i == 0 ? p.X : (i == 1 ? p.Y : p.Z)) = integer32(v); });
+        int32_t *const axis[3] = {&p.X, &p.Y, &p.Z};
+        items(a[4], 3, "grid must be (X, Y, Z)", [&](Py_ssize_t i, PyObject *v) { *axis[i] = integer32(v); });
         p.reduce = integer32(a[5]), p.kernel = integer32(a[8]), p.out_dtype = FLASHBEV_F32;
         tune(p.tune, a[9]);
         const StreamArg stream(a[10]);
@@ -357,9 +362,11 @@ PyObject *py_sca(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return guarded([&]() -> PyObject * {
         need_args(n, 12);
-        const at::Tensor &v = tensor(a[0], "value"), &m = tensor(a[2], "lidar2img"), &o = tensor(a[3], "offsets"), &w = tensor(a[4], "weights");
+        const at::Tensor &v = tensor(a[0], "value"), &m = tensor(a[2], "lidar2img");
+        const at::Tensor &o = tensor(a[3], "offsets"), &w = tensor(a[4], "weights");
         for (const at::Tensor *t : {&m, &o, &w})
-            if (!t->is_cuda() || t->scalar_type() != at::kFloat || !t->is_contiguous()) value_error("sca needs contiguous CUDA float32 tensors");
+            if (!t->is_cuda() || t->scalar_type() != at::kFloat || !t->is_contiguous())
+                value_error("sca needs contiguous CUDA float32 tensors");
         if (!v.is_cuda() || !v.is_contiguous() || (v.scalar_type() != at::kFloat && v.scalar_type() != at::kBFloat16))
             value_error("value must be a contiguous CUDA float32 or bfloat16 tensor");
         if (v.dim() != 5 || w.dim() != 5) value_error("value and weights must have five dimensions");
@@ -380,7 +387,8 @@ PyObject *py_sca(PyObject *, PyObject *const *a, Py_ssize_t n)
         });
         if (hw.size() < 2 * (size_t)p.L) value_error("level_hw must have an entry per level");
         geometry(p, a[5], a[6]);
-        items(a[7], 3, "grid must be (X, Y, Zref)", [&](Py_ssize_t i, PyObject *x) { (i == 0 ? p.X : (i == 1 ? p.Y : p.Zref)) = integer32(x); });
+        int32_t *const axis[3] = {&p.X, &p.Y, &p.Zref};
+        items(a[7], 3, "grid must be (X, Y, Zref)", [&](Py_ssize_t i, PyObject *x) { *axis[i] = integer32(x); });
         p.chunk_records = cut_integer32(a[11]);
         const StreamArg stream(a[10]);
         at::Tensor out;
