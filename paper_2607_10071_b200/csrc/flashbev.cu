@@ -382,12 +382,14 @@ __global__ void __launch_bounds__(256) vt_per_output_nchw_kernel(const KParams p
 //      coalesced streaming loads in the order the offsets and weights are stored -- into tap records
 //      {index of the upper left tap, 4 weights} in shared memory: attention weight x bilinear weight; the 2 x 2 block
 //      of taps is moved inside the map and the taps outside of it weigh 0 (zero padding without predicates).
-//      The other three taps are one texel and one row further (20 bytes per record: with all four indices, 32 bytes,
-//      the records were a third of the L1 data pipe's wavefronts, the unit that bounds this kernel: 371 -> 365 us at
-//      BEVFormer-base sizes);
+//      The other three taps are one texel and one row further (20 bytes per record, not 32 with all four indices:
+//      27 -> 22 M of the L1 data pipe's wavefronts, 371 -> 365 us at BEVFormer-base sizes);
 //   3. the lanes of a head (head_dim / 4 lanes, 16 bytes of the head's channels each) walk the head's
 //      records: four 128-bit loads and packed fp32 FMAs per record.
 // No per-camera, BEV-shaped tensor (reference points, masks, sampling locations) ever exists in memory.
+// At those sizes in fp32 no unit is at its limit: L1 data pipe 69 %, L2 58 %, issue slots 49 %, L2 to L1 39 % (5.1 GB, 18 % of
+// the tap sectors hit in L1).  The 19 resident warps of an SM spend nearly half of their time on taps that come from L2 (long
+// scoreboard: 4.4 of the 9.7 warp cycles per issued instruction).
 
 constexpr int kScaMaxLevels = 8;
 constexpr int kScaMaxChunkPoints = 32;  // sampling points per chunk (bit mask of visible points)
@@ -637,15 +639,16 @@ __global__ void __launch_bounds__(128, V == 1 && BF16 ? 7 : (V <= 2 ? 5 : 3)) sc
 
 // ------------------------------------------------------------------------------------------
 // Channel-planar features [planes][C][HW] -> channels last [planes][HW][Cpad] (T: 2- or 4-byte elements, Cpad: C rounded up to the
-// E elements of 16 bytes, the tail zero).  Bound by memory: a thread reads 16 bytes of E channel rows, transposes the E x E block in registers
-// (bf16: 32 byte permutes) and writes 16 bytes of E texels.  A warp covers 4 E channels x 8 E texels, so it reads whole
-// 128-byte lines and writes 64-byte pieces.  ALIGNED: HW is a multiple of E and the base is 16-byte aligned; otherwise the rows
-// are read element by element (they hit L1).  Measured on 6 x 128 x 64 x 176 bf16 (17 MB): 25 us with a 32 x 32 shared-memory
+// E elements of 16 bytes, the tail zero).  Bound by memory: a thread reads 16 bytes of E channel rows, transposes the E x E block
+// in registers (bf16: 32 byte permutes) and writes 16 bytes of E texels.  A warp covers 4 E channels x 8 E texels, so it reads
+// whole 128-byte lines and writes 64-byte pieces.  ALIGNED: HW is a multiple of E and the base is 16-byte aligned; otherwise the
+// rows are read element by element (they hit L1).  Measured on 6 x 128 x 64 x 176 bf16 (17 MB): 25 us with a 32 x 32 shared-memory
 // tile of 2-byte accesses, 7.6 us now.
 template <typename T, bool ALIGNED>
 __global__ void __launch_bounds__(256) nchw_to_nhwc_kernel(const T *__restrict__ in, T *__restrict__ out, int C, int Cpad, int HW)
 {
     constexpr int E = 16 / (int)sizeof(T);
+    using Bits = typename std::conditional<sizeof(T) == 2, uint16_t, uint32_t>::type;
     asm volatile("griddepcontrol.launch_dependents;");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int hw0 = (blockIdx.x * 8 + warp) * (8 * E) + (lane >> 2) * E, c0 = (blockIdx.y * 4 + (lane & 3)) * E;
@@ -664,7 +667,8 @@ __global__ void __launch_bounds__(256) nchw_to_nhwc_kernel(const T *__restrict__
         for (int i = 0; i < E; ++i) {
             uint32_t e[E];
 #pragma unroll
-            for (int j = 0; j < E; ++j) e[j] = c0 + i < C && hw0 + j < HW ? (uint32_t)*reinterpret_cast<const typename std::conditional<sizeof(T) == 2, uint16_t, uint32_t>::type *>(src + (size_t)i * HW + j) : 0u;
+            for (int j = 0; j < E; ++j)
+                e[j] = c0 + i < C && hw0 + j < HW ? (uint32_t)*reinterpret_cast<const Bits *>(src + (size_t)i * HW + j) : 0u;
 #pragma unroll
             for (int j = 0; j < 4; ++j) r[i][j] = sizeof(T) == 2 ? e[(2 * j) % E] | (e[(2 * j + 1) % E] << 16) : e[j % E];
         }
@@ -675,8 +679,9 @@ __global__ void __launch_bounds__(256) nchw_to_nhwc_kernel(const T *__restrict__
         uint4 v;
         if (sizeof(T) == 2) {
             const unsigned sel = (j & 1) ? 0x7632u : 0x5410u;
-            v.x = __byte_perm(r[0][j / 2 % 4], r[1][j / 2 % 4], sel), v.y = __byte_perm(r[2][j / 2 % 4], r[3][j / 2 % 4], sel);
-            v.z = __byte_perm(r[4 % E][j / 2 % 4], r[5 % E][j / 2 % 4], sel), v.w = __byte_perm(r[6 % E][j / 2 % 4], r[7 % E][j / 2 % 4], sel);
+            const int q = j / 2 % 4;
+            v.x = __byte_perm(r[0][q], r[1][q], sel), v.y = __byte_perm(r[2][q], r[3][q], sel);
+            v.z = __byte_perm(r[4 % E][q], r[5 % E][q], sel), v.w = __byte_perm(r[6 % E][q], r[7 % E][q], sel);
         } else {
             v = make_uint4(r[0][j % 4], r[1][j % 4], r[2][j % 4], r[3][j % 4]);
         }
@@ -685,10 +690,11 @@ __global__ void __launch_bounds__(256) nchw_to_nhwc_kernel(const T *__restrict__
 }
 
 // Channels-last rows of C elements -> rows of `vecs` 16-byte vectors, the tail zero (T: 2- or 4-byte elements; `total` vectors
-// per batch element, blockIdx.y).  One vector per thread; the reads of a warp are adjacent elements (whole lines over the E loads).  5 x 29 x 77 rows of 82 fp32: 9.1 us with a
-// 64-bit division per element, 4.3 us now.
+// per batch element, blockIdx.y).  One vector per thread; the reads of a warp are adjacent elements (whole lines over the E
+// loads).  5 x 29 x 77 rows of 82 fp32: 9.1 us with a 64-bit division per element, 4.3 us now.
 template <typename T>
-__global__ void __launch_bounds__(256) pad_channels_kernel(const T *__restrict__ in, uint4 *__restrict__ out, unsigned total, int C, unsigned vecs)
+__global__ void __launch_bounds__(256) pad_channels_kernel(const T *__restrict__ in, uint4 *__restrict__ out, unsigned total, int C,
+                                                           unsigned vecs)
 {
     constexpr int E = 16 / (int)sizeof(T);
     asm volatile("griddepcontrol.launch_dependents;");
@@ -871,9 +877,10 @@ int padded_channels(const flashbev_vt_params *p)
 
 // Bytes of the channels-last copy of NCHW features (0: the call takes no scratch).  Channel counts that are not whole vectors are
 // padded in the copy, from 12288 bins on.  Smaller grids ask for no scratch and run in one launch of the generic kernel: that is
-// the contract of flashbev_workspace_bytes, kept for the callers that rely on it and not for speed.  The copy and the tiled kernel win on both sides of the
-// line (N = 6, generic / tiled): 97 bf16 channels of 29 x 77, 50 x 50 x 4 bins 37.7 / 14.8 us, 64 x 48 x 4 33.7 / 14.8, 64 x 64 x 8
-// 50.9 / 18.1; 30 fp32 of 16 x 44, 34.7 / 9.3, 31.7 / 9.2, 41.2 / 10.2; 82 fp32 of 32 x 88, 44.6 / 16.8, 35.2 / 17.1, 59.3 / 23.9.
+// the contract of flashbev_workspace_bytes, kept for the callers that rely on it and not for speed.  The copy and the tiled
+// kernel win on both sides of the line (N = 6, generic / tiled): 97 bf16 channels of 29 x 77, 50 x 50 x 4 bins 37.7 / 14.8 us,
+// 64 x 48 x 4 33.7 / 14.8, 64 x 64 x 8 50.9 / 18.1; 30 fp32 of 16 x 44, 34.7 / 9.3, 31.7 / 9.2, 41.2 / 10.2; 82 fp32 of 32 x 88,
+// 44.6 / 16.8, 35.2 / 17.1, 59.3 / 23.9.
 size_t nchw_copy_bytes(const flashbev_vt_params *p)
 {
     if (p->layout != FLASHBEV_NCHW) return 0;
@@ -1152,8 +1159,10 @@ flashbev_status launch_nchw_tiled(const flashbev_vt_params *p, cudaStream_t stre
         using T = typename std::remove_pointer<decltype(elem)>::type;
         kernel<<<grid, dim3(256), 0, stream>>>(static_cast<const T *>(p->features), static_cast<T *>(p->workspace), p->C, q.C, HW);
     };
-    if (E == 8) aligned ? copy(nchw_to_nhwc_kernel<uint16_t, true>, (uint16_t *)nullptr) : copy(nchw_to_nhwc_kernel<uint16_t, false>, (uint16_t *)nullptr);
-    else aligned ? copy(nchw_to_nhwc_kernel<float, true>, (float *)nullptr) : copy(nchw_to_nhwc_kernel<float, false>, (float *)nullptr);
+    if (E == 8 && aligned) copy(nchw_to_nhwc_kernel<uint16_t, true>, (uint16_t *)nullptr);
+    else if (E == 8) copy(nchw_to_nhwc_kernel<uint16_t, false>, (uint16_t *)nullptr);
+    else if (aligned) copy(nchw_to_nhwc_kernel<float, true>, (float *)nullptr);
+    else copy(nchw_to_nhwc_kernel<float, false>, (float *)nullptr);
     if (cudaGetLastError() != cudaSuccess) return FLASHBEV_CUDA_ERROR;
     const flashbev_status st = launch_tiled(&q, stream, accumulate, 1, p->C);
     if (st == FLASHBEV_OK) t_last_kernel = p->feat_dtype == FLASHBEV_BF16 ? "tiled_bf16_nchw" : "tiled_f32_nchw";
@@ -1180,11 +1189,11 @@ flashbev_status launch_padded_tiled(const flashbev_vt_params *p, cudaStream_t st
     const unsigned total = (unsigned)p->N * p->feat_h * p->feat_w * vecs;  // < 2^31 (pad_copy_bytes)
     const dim3 blocks((total + 255) / 256, (unsigned)p->B);
     if (p->feat_dtype == FLASHBEV_BF16)
-        pad_channels_kernel<uint16_t><<<blocks, 256, 0, stream>>>(static_cast<const uint16_t *>(p->features), static_cast<uint4 *>(p->workspace),
-                                                                  total, p->C, (unsigned)vecs);
+        pad_channels_kernel<uint16_t><<<blocks, 256, 0, stream>>>(static_cast<const uint16_t *>(p->features),
+                                                                  static_cast<uint4 *>(p->workspace), total, p->C, (unsigned)vecs);
     else
-        pad_channels_kernel<float><<<blocks, 256, 0, stream>>>(static_cast<const float *>(p->features), static_cast<uint4 *>(p->workspace),
-                                                               total, p->C, (unsigned)vecs);
+        pad_channels_kernel<float><<<blocks, 256, 0, stream>>>(static_cast<const float *>(p->features),
+                                                               static_cast<uint4 *>(p->workspace), total, p->C, (unsigned)vecs);
     if (cudaGetLastError() != cudaSuccess) return FLASHBEV_CUDA_ERROR;
     const flashbev_status st = launch_tiled(&q, stream, accumulate, 2, p->C);
     if (st == FLASHBEV_OK) t_last_kernel = p->feat_dtype == FLASHBEV_BF16 ? "tiled_bf16_padded" : "tiled_f32_padded";
@@ -1350,8 +1359,10 @@ flashbev_status flashbev_sampling_vt_backward(const flashbev_vt_backward_params 
     dim3 grid;
     size_t smem;
     p.tune[3] = (p.tune[3] & ~0xf) | 4;  // the backward instances are built for 4 warps per CTA
-    // (measured) the scatter is bound by reductions on hot L2 sectors: small blocks in single-row bands spread them
-    // best (7-9 % over the forward's defaults)
+    // (measured) the scatter is bound by the reductions that an SM hands to the crossbar: the request port is busy in 77 % of an
+    // SM's active cycles (93 % on the busiest) with 11.5 M sectors on 200 x 200 x 8, C = 80, and in 81 % (99 %) with 22 M on a
+    // calibrated rig, C = 128; the L2's reduction units in 36 and 43 % (busiest slice 42 and 49 %).  Small blocks in single-row
+    // bands share the work out best (7-9 % over the forward's defaults).
     if ((long long)p.B * p.X * p.Y >= 16384) {  // (small grids: the forward's defaults)
         if (!(p.tune[3] & 0xff0)) p.tune[3] |= (1 << 4) | (2 << 8);
         if (!(p.tune[3] & 0xc0000)) p.tune[3] |= 0x40000;
