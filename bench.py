@@ -40,7 +40,7 @@ MIN_LAUNCHES_PER_STEP = 64
 # launches taken from the middle of a step of rotating frames -- the regime that is timed -- summarised under
 # profiles/vt_tiled_kernel_<workload>.md.  The output of a launch is still partly in the 126 MB L2 when its kernel
 # ends, so these figures can lie below the algorithmic bytes: see `traffic_note` in the JSON line.
-NCU_DRAM_TRAFFIC = {"tiny": 0.342e6, "representative": 4.78e6, "half_taller": 8.20e6, "long_range": 41.00e6, "high_res": 21.45e6}
+NCU_DRAM_TRAFFIC = {"tiny": 0.329e6, "representative": 4.77e6, "half_taller": 8.11e6, "long_range": 40.56e6, "high_res": 21.45e6}
 TRAFFIC_NOTE = ("dram__bytes_read.sum + dram__bytes_write.sum of one launch captured in the middle of a rotating-frame "
                 "step (ncu, one pass); part of a launch's output is written back from L2 after its kernel ends, so the "
                 "figure can be below the algorithmic bytes")
@@ -503,7 +503,7 @@ def full_block(torch, w, args, device, rank, barrier, steps, warmup, world, redu
                      "algorithmic_bytes_per_launch": w.unique_bytes, "frac_of_8TBs_nominal": achieved / 8000.0,
                      "target_frac": 0.5, "target_met": bool(achieved / peak >= 0.5),
                      "what_binds": "not HBM: a cached gather (features stay in L2); instruction issue and the L1 data "
-                                   "pipe set the time, see profiles/"},
+                                   "pipe are the busiest units, see profiles/"},
         "peak_mb": {"workspace_allocated_by_call": workspace / 1e6, "output": w.output_bytes / 1e6,
                     "inputs_plus_output": w.unique_bytes / 1e6},
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": e2e["h2d"], "d2h_bytes_per_step": e2e["d2h"],
