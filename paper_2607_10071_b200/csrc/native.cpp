@@ -265,6 +265,8 @@ PyObject *py_sampling_vt_backward(PyObject *, PyObject *const *a, Py_ssize_t n)
         const at::Tensor &g = tensor(a[0], "grad_out"), &m = tensor(a[1], "lidar2img");
         if (!g.is_cuda() || g.scalar_type() != at::kFloat || !g.is_contiguous())
             value_error("grad_out must be a contiguous CUDA float32 tensor");
+        if (!m.is_cuda() || m.scalar_type() != at::kFloat || !m.is_contiguous())
+            value_error("lidar2img must be a contiguous CUDA float32 tensor");
         if (g.dim() != 4) value_error("grad_out must have four dimensions");
         flashbev_vt_backward_params p = {};
         p.struct_size = sizeof(p);

@@ -21,6 +21,15 @@ def test_rig_with_too_few_dimensions_is_an_index_error():
         fb.sampling_vt_backward(grad, rig, (8, 8), (64, 64), RANGE, (5, 6, 4))
 
 
+def test_backward_refuses_a_rig_that_its_kernel_cannot_read():
+    """As the other calls do: host memory, other number types, strides."""
+    torch = pytest.importorskip("torch")
+    grad, rig = _fake_cuda(1, 5, 6, 8), _fake_cuda(1, 2, 4, 4)
+    for bad in (torch.zeros((1, 2, 4, 4)), rig.to(torch.float64), rig.transpose(2, 3)):
+        with pytest.raises(ValueError, match="lidar2img"):
+            fb.sampling_vt_backward(grad, bad, (8, 8), (64, 64), RANGE, (5, 6, 4))
+
+
 @pytest.mark.gpu
 def test_numbers_are_converted_as_python_converts_them():
     """bev_range by float(), hints by int(), level_hw as numpy casts it; the backward reads the height bins only from the grid."""
