@@ -369,8 +369,9 @@ __global__ void __launch_bounds__(256) vt_per_output_nchw_kernel(const KParams p
 }
 
 // ------------------------------------------------------------------------------------------
-// Kernel 2: tiled (forward and backward), see vt_tiled.cuh
+// Kernel 2: tiled (forward and the scatter form of the backward), see vt_tiled.cuh; the texel-side backward, see vt_backward.cuh
 #include "vt_tiled.cuh"
+#include "vt_backward.cuh"
 
 // ------------------------------------------------------------------------------------------
 // Kernel 3: FlashSCA -- spatial cross-attention with on-the-fly projection (paper Sec. 4.4).  One warp per
@@ -1135,6 +1136,89 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
     return e == cudaSuccess ? FLASHBEV_OK : FLASHBEV_CUDA_ERROR;
 }
 
+// Chooses the tiles and the grid of the texel-side backward kernel.  NT: channels per warp / 8.
+flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, int &NT, dim3 &grid, size_t &smem)
+{
+    q = {};
+    q.k = base_params(p);
+    const int ch_tiles = (p->C + 79) / 80;
+    NT = ((p->C + ch_tiles - 1) / ch_tiles + 15) / 16 * 2;  // (instances for every other NT)
+    q.row_tiles = std::min(kBwdMaxTiles, (p->feat_h + kBwdRows - 1) / kBwdRows);
+    q.ch_tiles = std::min(ch_tiles, kBwdMaxWarps / q.row_tiles);
+    q.groups = std::max(1, 4 / (q.row_tiles * q.ch_tiles));
+    const int rows = q.row_tiles * kBwdRows, channels = 8 * NT * q.ch_tiles;
+    const int cblocks = (p->C + channels - 1) / channels, rblocks = (p->feat_h + rows - 1) / rows;
+    const double columns = (double)p->B * p->N * p->feat_w * cblocks * rblocks;
+    // One CTA per column stores its sums, without a memset before and reductions after it.  Where that leaves SMs idle with long
+    // lists, two share a column.  One / two / three CTAs per column, us: 176 columns, 18 k cells, C = 96 23 / 20 / 23; 258, 28 k,
+    // C = 48 54 / 39 / 37; 276, 48 k, C = 32 29 / 26 / 32; but 252, 12 k, C = 96 17 / 29 / 37, 290, 12 k, C = 48 28 / 27 / 31, and
+    // 528, 40 k, C = 80 33 / 37 / 39.
+    q.slices = columns <= 2.0 * sm_count() && (double)p->X * p->Y > 100.0 * p->N * p->feat_w ? 2 : 1;
+    q.exclusive = q.slices == 1;
+    smem = bwd_smem_layout(nullptr, nullptr, p->N, q.row_tiles, q.ch_tiles, q.groups, NT, p->reduce);
+    const double blocks = (double)p->B * p->N * p->feat_w * q.slices;
+    if (blocks > 2147483647.0 || cblocks > 65535 || rblocks > 65535 || smem > 200 * 1024) return FLASHBEV_UNSUPPORTED;
+    grid = dim3((unsigned)blocks, (unsigned)cblocks, (unsigned)rblocks);
+    return FLASHBEV_OK;
+}
+
+template <int NT>
+cudaError_t launch_backward(const BwdParams &q, dim3 grid, size_t smem, cudaStream_t stream)
+{
+    const auto kernel = q.k.reduce == FLASHBEV_REDUCE_SUM ? vt_texel_backward_kernel<NT, true> : vt_texel_backward_kernel<NT, false>;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    kernel<<<grid, dim3((unsigned)(q.row_tiles * q.ch_tiles * q.groups * 32)), smem, stream>>>(q);
+    return cudaSuccess;
+}
+
+// Which of the two backward kernels takes a call: the texel-side one, but not
+// - with hints, which are launch geometry of the scatter;
+// - with few channels over many cells: its geometry is made for every texel column that a cell reaches (scatter / texel side, us,
+//   C = 32, N = 6 tilted cameras with 57 x 50 maps, 2 x 58 k cells 118 / 163; N = 8, 134 k cells 94 / 139; but level cameras
+//   99 / 60 with 62 k cells, and with fewer cells 32 / 33 (24 k, tilted), 22 / 16 (14 k, level), 41 / 29 (44 k, level));
+// - with more than 64 height bins, each of which it projects (the scatter solves for intervals).
+// From 48 channels on it wins on all of 33 measured calls by up to 2.8x (200 x 200 x 8, C = 80 92 / 33, C = 128 on tilted cameras
+// 144 / 90), but for one draw (30 / 31).
+bool backward_by_texel(const flashbev_vt_params *p)
+{
+    for (int t : p->tune)
+        if (t) return false;
+    if (p->Z > 64) return false;
+    return p->C > 40 || (double)p->X * p->Y <= 120.0 * p->N * p->feat_w;
+}
+
+flashbev_status launch_texel_backward(const flashbev_vt_params *p, const float *grad_out, float *grad_features, cudaStream_t stream)
+{
+    BwdParams q;
+    int NT;
+    dim3 grid;
+    size_t smem;
+    const flashbev_status st = configure_backward(p, q, NT, grid, smem);
+    if (st != FLASHBEV_OK) return st;
+    q.k.feat = nullptr, q.k.out = nullptr, q.k.count_out = nullptr;
+    q.k.gout = grad_out, q.k.gfeat = grad_features;
+    if (!q.exclusive) {
+        const size_t bytes = (size_t)p->B * p->N * p->feat_h * p->feat_w * p->C * sizeof(float);
+        if (cudaMemsetAsync(grad_features, 0, bytes, stream) != cudaSuccess) {
+            cudaGetLastError();
+            return FLASHBEV_CUDA_ERROR;
+        }
+    }
+    cudaError_t e;
+    if (NT <= 2) e = launch_backward<2>(q, grid, smem, stream);
+    else if (NT <= 4) e = launch_backward<4>(q, grid, smem, stream);
+    else if (NT <= 6) e = launch_backward<6>(q, grid, smem, stream);
+    else if (NT <= 8) e = launch_backward<8>(q, grid, smem, stream);
+    else e = launch_backward<10>(q, grid, smem, stream);
+    if (e != cudaSuccess || cudaGetLastError() != cudaSuccess) return FLASHBEV_CUDA_ERROR;
+    t_last_launches = 1;
+    t_last_kernel = "tiled_bwd_texel";
+    return FLASHBEV_OK;
+}
+
 // NCHW tensors on the tiled kernel: features -> channels-last copy in the workspace, output written planar.
 flashbev_status launch_nchw_tiled(const flashbev_vt_params *p, cudaStream_t stream, bool accumulate)
 {
@@ -1354,12 +1438,17 @@ flashbev_status flashbev_sampling_vt_backward(const flashbev_vt_backward_params 
     if (((uintptr_t)q->grad_out % 16) || ((uintptr_t)q->grad_features % 16) || ((uintptr_t)q->lidar2img % 4))
         return FLASHBEV_MISALIGNED;
     if (q->C % 4 || !tiled_applicable(&p)) return FLASHBEV_UNSUPPORTED;
+    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+    if (backward_by_texel(&p)) {
+        st = launch_texel_backward(&p, q->grad_out, q->grad_features, stream);
+        if (st != FLASHBEV_UNSUPPORTED) return st;
+    }
     KParams k;
     int V, warps;
     dim3 grid;
     size_t smem;
     p.tune[3] = (p.tune[3] & ~0xf) | 4;  // the backward instances are built for 4 warps per CTA
-    // (measured) the scatter is bound by the reductions that an SM hands to the crossbar: the request port is busy in 77 % of an
+    // the scatter (measured): it is bound by the reductions that an SM hands to the crossbar: the request port is busy in 77 % of an
     // SM's active cycles (93 % on the busiest) with 11.5 M sectors on 200 x 200 x 8, C = 80, and in 81 % (99 %) with 22 M on a
     // calibrated rig, C = 128; the L2's reduction units in 36 and 43 % (busiest slice 42 and 49 %).  Small blocks in single-row
     // bands share the work out best (7-9 % over the forward's defaults).
@@ -1370,7 +1459,6 @@ flashbev_status flashbev_sampling_vt_backward(const flashbev_vt_backward_params 
     if ((st = configure_tiled(&p, k, V, warps, grid, smem, false, true)) != FLASHBEV_OK) return st;
     k.feat = nullptr, k.out = nullptr, k.count_out = nullptr;
     k.gout = q->grad_out, k.gfeat = q->grad_features;
-    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const size_t bytes = (size_t)q->B * q->N * q->feat_h * q->feat_w * q->C * sizeof(float);
     if (cudaMemsetAsync(q->grad_features, 0, bytes, stream) != cudaSuccess) {
         cudaGetLastError();

@@ -1,0 +1,95 @@
+"""The texel-side backward kernel at the sizes where it can go wrong: edges of its row tiles (16 and 64 rows), channel tiles
+(80 channels, 8 per fragment) and channel blocks, maps of one texel, one and two CTAs per texel column, and gradients that are
+not finite.  Tolerances are those of the backward's other tests (`test_gpu_backward`), the same bounds for both kernels."""
+import numpy as np
+import pytest
+
+from paper_2607_10071_b200 import binding as fb
+from paper_2607_10071_b200 import build as fbuild
+from paper_2607_10071_b200 import workloads as wl
+from tests.test_gpu_backward import check, run_backward
+
+pytestmark = pytest.mark.gpu
+SUM, MEAN, EQ1 = 0, 1, 2
+SCATTER = (0, 0, 16, 0)  # hints select the scatter kernel
+
+
+def workload(name, C, feat, grid, general=True, B=1, N=6, xy=25.0, reduce=0):
+    return wl.Workload(name, 9100 + C, B, N, C, "f32", feat, (feat[0] * 8, feat[1] * 8), grid, (-xy, xy, -xy, xy, -4.0, 3.0), reduce,
+                       general_pose=general)
+
+
+@pytest.mark.parametrize("feat", [(1, 1), (1, 9), (15, 7), (16, 12), (17, 30), (32, 20), (33, 11), (64, 10), (65, 10), (130, 6)])
+@pytest.mark.parametrize("reduce", [SUM, MEAN, EQ1])
+def test_row_tiles(oracle, feat, reduce):
+    for general in (False, True):
+        w = workload("rows", 44, feat, (37, 41, 9), general)
+        assert "texel" in check(oracle, w, wl.make_inputs(w).lidar2img, reduce, seed=feat[0])
+
+
+@pytest.mark.parametrize("C", [4, 8, 12, 16, 32, 36, 80, 84, 96, 128, 132, 160, 164, 320, 324, 644])
+def test_channel_tiles(oracle, C):
+    w = workload("channels", C, (18, 26), (29, 33, 6), B=2, N=3)
+    assert "texel" in check(oracle, w, wl.make_inputs(w).lidar2img, C // 4 % 3, seed=C)
+
+
+@pytest.mark.parametrize("Z", [1, 2, 3, 5, 63, 64])
+def test_height_bins(oracle, Z):
+    w = workload("bins", 48, (20, 24), (31, 30, Z), N=5)
+    for reduce in (SUM, MEAN, EQ1):
+        assert "texel" in check(oracle, w, wl.make_inputs(w).lidar2img, reduce, seed=Z)
+
+
+@pytest.mark.parametrize("general", [False, True])
+def test_two_blocks_per_column_and_a_full_list(oracle, general):
+    """Few texel columns over many cells: two CTAs share a column, and its cells do not fit the list at once."""
+    w = workload("long_lists", 48, (24, 10), (220, 190, 4), general, N=2, xy=40.0)
+    for reduce in (SUM, EQ1):
+        assert "texel" in check(oracle, w, wl.make_inputs(w).lidar2img, reduce)
+
+
+def test_many_cameras_see_every_cell(oracle):
+    w = workload("cameras", 40, (16, 20), (24, 22, 7), N=33)
+    inp = wl.make_inputs(w)
+    inp.lidar2img[:] = inp.lidar2img[:, :1]
+    for reduce in (SUM, MEAN, EQ1):
+        assert "texel" in check(oracle, w, inp.lidar2img, reduce)
+
+
+@pytest.mark.parametrize("shared", [False, True])
+def test_gradients_that_are_not_finite(shared):
+    """Infinite and NaN output gradients reach the texels that their cell weighs and no others, as in the scatter."""
+    w = workload("nonfinite", 44, (24, 10), (220, 190, 4), N=2) if shared else workload("nonfinite", 84, (33, 20), (40, 40, 6))
+    m = wl.make_inputs(w).lidar2img
+    rng = np.random.default_rng(5)
+    G = rng.standard_normal((w.B,) + tuple(w.grid[:2]) + (w.C,)).astype(np.float32)
+    for value, cells in ((np.inf, 3), (-np.inf, 3), (np.nan, 2), (3.4e38, 2)):
+        for _ in range(cells):
+            G[0, rng.integers(w.grid[0]), rng.integers(w.grid[1]), rng.integers(w.C)] = value
+    for reduce in (SUM, MEAN, EQ1):
+        got, name = run_backward(w, m, G, reduce)
+        ref, other = run_backward(w, m, G, reduce, SCATTER)
+        assert "texel" in name and "texel" not in other
+        assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isposinf(got), np.isposinf(ref))
+        assert np.array_equal(np.isneginf(got), np.isneginf(ref)) and not np.isfinite(ref).all()
+        ok = np.isfinite(ref)
+        # two fp32 sums of the same numbers: 2e-6 of the result each (test_gpu_backward), per channel (the large value stands alone)
+        err = np.where(ok, got, 0.0).astype(np.float64) - np.where(ok, ref, 0.0)
+        assert np.all(np.sqrt((err ** 2).sum((0, 1, 2, 3))) <= 4e-6 * np.sqrt((np.where(ok, ref, 0.0).astype(np.float64) ** 2).sum((0, 1, 2, 3))))
+
+
+@pytest.mark.parametrize("reduce", [SUM, MEAN, EQ1])
+def test_makes_no_out_of_range_index(reduce):
+    import torch
+    lib = fb.load_library(fbuild.build(debug_bounds=True))
+    dev = torch.device("cuda:0")
+    for C, feat, grid, N in ((44, (65, 10), (37, 41, 9), 6), (132, (17, 30), (64, 48, 5), 4), (48, (24, 10), (220, 190, 4), 2)):
+        w = workload("bounds", C, feat, grid, N=N)
+        m = torch.from_numpy(wl.make_inputs(w).lidar2img).to(dev)
+        g = torch.randn((1,) + tuple(grid[:2]) + (C,), device=dev)
+        g[0, 3, 3, 1] = float("inf")
+        out, err = torch.empty((1, N) + feat + (C,), device=dev), torch.zeros(1, dtype=torch.int32, device=dev)
+        p = fb.make_backward_params(g.data_ptr(), m.data_ptr(), 1, N, C, feat, w.img_hw, w.bev_range, grid, reduce, out.data_ptr(),
+                                    debug_error_word=err.data_ptr())
+        fb.flashbev_sampling_vt_backward(p, torch.cuda.current_stream().cuda_stream, library=lib)
+        assert err.item() == 0 and lib.flashbev_last_kernel_name() == b"tiled_bwd_texel"
