@@ -49,6 +49,7 @@ struct KParams {
     int out_c;                  // ... channels of the output (the kernel's C may be padded)
     size_t out_bs, out_cells, out_chs;  // ... element strides of batch element, cell and channel
     int pdl;                    // host only: launch the forward with programmatic stream serialization
+    int tell_late;              // another kernel of the same call follows: start it only after the wait for what ran before
     int accumulate;             // add the result to the fp32 output instead of overwriting it (multi-resolution levels)
     double sx, sy;              // image px -> feature px
     double x_min, dx, y_min, dy, z_min, dz;
@@ -650,6 +651,8 @@ __global__ void __launch_bounds__(256) nchw_to_nhwc_kernel(const T *__restrict__
 {
     constexpr int E = 16 / (int)sizeof(T);
     using Bits = typename std::conditional<sizeof(T) == 2, uint16_t, uint32_t>::type;
+    // (the tiled kernel after this one reads its matrices at once: see there)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int hw0 = (blockIdx.x * 8 + warp) * (8 * E) + (lane >> 2) * E, c0 = (blockIdx.y * 4 + (lane & 3)) * E;
@@ -698,6 +701,7 @@ __global__ void __launch_bounds__(256) pad_channels_kernel(const T *__restrict__
                                                            unsigned vecs)
 {
     constexpr int E = 16 / (int)sizeof(T);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;");
     const unsigned i = blockIdx.x * 256u + threadIdx.x;
     if (i >= total) return;
@@ -959,6 +963,8 @@ cudaError_t launch_tiled_warps(int warps, const KParams &k, dim3 grid, size_t sm
     }
 }
 
+int use_pdl() { return getenv("FLASHBEV_NO_PDL") ? 0 : 1; }
+
 // Chooses the channel mapping, super-block shape, run length, list size and grid of the tiled kernel.
 flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V, int &warps, dim3 &grid, size_t &smem,
                                 bool accumulate = false, bool backward = false, bool planar = false)
@@ -1102,8 +1108,8 @@ flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V,
 
 // scalar_out: 0 vector stores into channels-last rows; 1 planar output [B][out_c][X][Y]; 2 channels-last rows of out_c
 // channels (the kernel's own C may be padded)
-flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, bool accumulate = false, int scalar_out = 0,
-                             int out_c = 0)
+flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, bool accumulate = false, bool tell_late = false,
+                             int scalar_out = 0, int out_c = 0)
 {
     KParams k;
     int V, warps;
@@ -1117,7 +1123,8 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
         if (scalar_out == 1) k.out_c = out_c, k.out_bs = plane * out_c, k.out_cells = 1, k.out_chs = plane;
         if (scalar_out == 2) k.out_c = out_c, k.out_bs = plane * out_c, k.out_cells = out_c, k.out_chs = 1;
     }
-    k.pdl = getenv("FLASHBEV_NO_PDL") ? 0 : 1;
+    k.pdl = use_pdl();
+    k.tell_late = tell_late;
     const bool bf16 = p->feat_dtype == FLASHBEV_BF16;
     cudaError_t e;
     static const char *const names[2][4] = {{"tiled_f32_v1", "tiled_f32_v2", "tiled_f32_v3", "tiled_f32_v4"},
@@ -1219,6 +1226,19 @@ flashbev_status launch_texel_backward(const flashbev_vt_params *p, const float *
     return FLASHBEV_OK;
 }
 
+// A copy kernel (256 threads), which waits for the kernel before it in the stream and then lets the tiled kernel start.
+template <typename... P, typename... A>
+void launch_copy(void (*kernel)(P...), dim3 grid, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid, cfg.blockDim = dim3(256), cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    if (use_pdl()) cfg.attrs = attr, cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // NCHW tensors on the tiled kernel: features -> channels-last copy in the workspace, output written planar.
 flashbev_status launch_nchw_tiled(const flashbev_vt_params *p, cudaStream_t stream, bool accumulate)
 {
@@ -1241,14 +1261,14 @@ flashbev_status launch_nchw_tiled(const flashbev_vt_params *p, cudaStream_t stre
     const dim3 grid((unsigned)((HW + 64 * E - 1) / (64 * E)), (unsigned)((q.C + 4 * E - 1) / (4 * E)), (unsigned)(p->B * p->N));
     auto copy = [&](auto kernel, auto *elem) {
         using T = typename std::remove_pointer<decltype(elem)>::type;
-        kernel<<<grid, dim3(256), 0, stream>>>(static_cast<const T *>(p->features), static_cast<T *>(p->workspace), p->C, q.C, HW);
+        launch_copy(kernel, grid, stream, static_cast<const T *>(p->features), static_cast<T *>(p->workspace), p->C, q.C, HW);
     };
     if (E == 8 && aligned) copy(nchw_to_nhwc_kernel<uint16_t, true>, (uint16_t *)nullptr);
     else if (E == 8) copy(nchw_to_nhwc_kernel<uint16_t, false>, (uint16_t *)nullptr);
     else if (aligned) copy(nchw_to_nhwc_kernel<float, true>, (float *)nullptr);
     else copy(nchw_to_nhwc_kernel<float, false>, (float *)nullptr);
     if (cudaGetLastError() != cudaSuccess) return FLASHBEV_CUDA_ERROR;
-    const flashbev_status st = launch_tiled(&q, stream, accumulate, 1, p->C);
+    const flashbev_status st = launch_tiled(&q, stream, accumulate, false, 1, p->C);
     if (st == FLASHBEV_OK) t_last_kernel = p->feat_dtype == FLASHBEV_BF16 ? "tiled_bf16_nchw" : "tiled_f32_nchw";
     return st;
 }
@@ -1273,20 +1293,22 @@ flashbev_status launch_padded_tiled(const flashbev_vt_params *p, cudaStream_t st
     const unsigned total = (unsigned)p->N * p->feat_h * p->feat_w * vecs;  // < 2^31 (pad_copy_bytes)
     const dim3 blocks((total + 255) / 256, (unsigned)p->B);
     if (p->feat_dtype == FLASHBEV_BF16)
-        pad_channels_kernel<uint16_t><<<blocks, 256, 0, stream>>>(static_cast<const uint16_t *>(p->features),
-                                                                  static_cast<uint4 *>(p->workspace), total, p->C, (unsigned)vecs);
+        launch_copy(pad_channels_kernel<uint16_t>, blocks, stream, static_cast<const uint16_t *>(p->features),
+                    static_cast<uint4 *>(p->workspace), total, p->C, (unsigned)vecs);
     else
-        pad_channels_kernel<float><<<blocks, 256, 0, stream>>>(static_cast<const float *>(p->features),
-                                                               static_cast<uint4 *>(p->workspace), total, p->C, (unsigned)vecs);
+        launch_copy(pad_channels_kernel<float>, blocks, stream, static_cast<const float *>(p->features),
+                    static_cast<uint4 *>(p->workspace), total, p->C, (unsigned)vecs);
     if (cudaGetLastError() != cudaSuccess) return FLASHBEV_CUDA_ERROR;
-    const flashbev_status st = launch_tiled(&q, stream, accumulate, 2, p->C);
+    const flashbev_status st = launch_tiled(&q, stream, accumulate, false, 2, p->C);
     if (st == FLASHBEV_OK) t_last_kernel = p->feat_dtype == FLASHBEV_BF16 ? "tiled_bf16_padded" : "tiled_f32_padded";
     return st;
 }
 
-flashbev_status run_device(const flashbev_vt_params *p, cudaStream_t stream, bool accumulate = false)
+// `level`, `levels`: of a pyramid; levels after the first add to the output
+flashbev_status run_device(const flashbev_vt_params *p, cudaStream_t stream, int level = 0, int levels = 1)
 {
     flashbev_status st;
+    const bool accumulate = level > 0;
     if (p->layout == FLASHBEV_NHWC && p->kernel != FLASHBEV_KERNEL_PER_OUTPUT && padded_tiled_applicable(p)) {
         st = launch_padded_tiled(p, stream, accumulate);
         if (st == FLASHBEV_OK) {
@@ -1315,7 +1337,7 @@ flashbev_status run_device(const flashbev_vt_params *p, cudaStream_t stream, boo
     }
     const bool tiled = p->kernel == FLASHBEV_KERNEL_TILED || (p->kernel == FLASHBEV_KERNEL_AUTO && tiled_applicable(p));
     if (tiled && !tiled_applicable(p)) return FLASHBEV_UNSUPPORTED;
-    st = tiled ? launch_tiled(p, stream, accumulate) : launch_per_output(p, stream, accumulate);
+    st = tiled ? launch_tiled(p, stream, accumulate, level == 0 && levels > 1) : launch_per_output(p, stream, accumulate);
     // AUTO: shapes the tiled kernel cannot be configured for (nothing was launched) go to the generic kernel
     if (tiled && st == FLASHBEV_UNSUPPORTED && p->kernel == FLASHBEV_KERNEL_AUTO) st = launch_per_output(p, stream, accumulate);
     if (st != FLASHBEV_OK) return st;
@@ -1495,7 +1517,7 @@ flashbev_status flashbev_sampling_vt_multires(const flashbev_vt_multires_params 
         if (tiled && !tiled_applicable(&lv[l])) return FLASHBEV_UNSUPPORTED;
     }
     for (int l = 0; l < q->levels; ++l)
-        if ((st = run_device(&lv[l], static_cast<cudaStream_t>(stream), l > 0)) != FLASHBEV_OK) return st;
+        if ((st = run_device(&lv[l], static_cast<cudaStream_t>(stream), l, q->levels)) != FLASHBEV_OK) return st;
     t_last_launches = q->levels;
     return FLASHBEV_OK;
 }
