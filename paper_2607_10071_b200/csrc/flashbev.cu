@@ -1172,7 +1172,9 @@ flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, in
 template <int NT>
 cudaError_t launch_backward(const BwdParams &q, dim3 grid, size_t smem, cudaStream_t stream)
 {
-    const auto kernel = q.k.reduce == FLASHBEV_REDUCE_SUM ? vt_texel_backward_kernel<NT, true> : vt_texel_backward_kernel<NT, false>;
+    const bool sum = q.k.reduce == FLASHBEV_REDUCE_SUM, full = q.k.C == (int)grid.y * q.ch_tiles * 8 * NT;
+    const auto kernel = sum ? (full ? vt_texel_backward_kernel<NT, true, true> : vt_texel_backward_kernel<NT, true, false>)
+                            : (full ? vt_texel_backward_kernel<NT, false, true> : vt_texel_backward_kernel<NT, false, false>);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1183,18 +1185,18 @@ cudaError_t launch_backward(const BwdParams &q, dim3 grid, size_t smem, cudaStre
 
 // Which of the two backward kernels takes a call: the texel-side one, but not
 // - with hints, which are launch geometry of the scatter;
-// - with few channels over many cells: its geometry is made for every texel column that a cell reaches (scatter / texel side, us,
-//   C = 32, N = 6 tilted cameras with 57 x 50 maps, 2 x 58 k cells 118 / 163; N = 8, 134 k cells 94 / 139; but level cameras
-//   99 / 60 with 62 k cells, and with fewer cells 32 / 33 (24 k, tilted), 22 / 16 (14 k, level), 41 / 29 (44 k, level));
-// - with more than 64 height bins, each of which it projects (the scatter solves for intervals).
-// From 48 channels on it wins on all of 33 measured calls by up to 2.8x (200 x 200 x 8, C = 80 92 / 33, C = 128 on tilted cameras
-// 144 / 90), but for one draw (30 / 31).
+// - with more than 64 height bins, each of which it projects (the scatter solves for intervals);
+// - with few channels, unless in SUM mode on few cells: it makes its geometry, and the mean modes their counts, for every texel
+//   column that a cell reaches, whatever the channels.  Scatter / texel side, us, C = 32, tilted cameras: Eq. 1 on 37 k cells 56 / 95,
+//   63 k 103 / 147; mean on 6 k 18 / 25, 10 k 23 / 25; SUM on 19 k 36 / 42, 28 k 64 / 59, but 6 k 16 / 12, 14 k 33 / 21, 9 k 23 / 17.
+// From 48 channels on it wins: 44 of 46 measured calls by up to 2.8x (geometric mean 1.55; 200 x 200 x 8, C = 80 92 / 33, C = 128 on
+// tilted cameras 143 / 87), the others 45 / 47 and 30 / 29.
 bool backward_by_texel(const flashbev_vt_params *p)
 {
     for (int t : p->tune)
         if (t) return false;
     if (p->Z > 64) return false;
-    return p->C > 40 || (double)p->X * p->Y <= 120.0 * p->N * p->feat_w;
+    return p->C > 40 || (p->reduce == FLASHBEV_REDUCE_SUM && (double)p->X * p->Y <= 50.0 * p->N * p->feat_w);
 }
 
 flashbev_status launch_texel_backward(const flashbev_vt_params *p, const float *grad_out, float *grad_features, cudaStream_t stream)

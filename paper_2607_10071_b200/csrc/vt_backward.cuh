@@ -22,9 +22,10 @@
 //
 // Why: the scatter hands two fp32 vector reductions per record to the crossbar -- 11.5 M sectors for a gradient of 0.17 M on
 // 200 x 200 x 8, C = 80 -- and is bound by the rate at which an SM can do that (92 us).  Here a texel leaves the SM once: 33 us;
-// 56 x 100 maps of tilted cameras, C = 128, Eq. 1: 144 -> 90 us.  What bounds it now: no unit (issue 34 %, tensor pipe 17 %); 16
+// 56 x 100 maps of tilted cameras, C = 128, Eq. 1: 144 -> 87 us.  What bounds it now: no unit (issue 34 %, tensor pipe 17 %); 16
 // warps per SM that wait at the barriers of a round, for grad_out and for chains of fp64 operations, in 0.9 to 2 waves of CTAs of
-// unequal size.  128 registers: with 80 (24 warps per SM) the spills cost more than the warps bring (calibrated 90 -> 110 us).
+// unequal size.  128 registers: with 80 (24 warps per SM) the spills cost more than the warps bring
+// (calibrated 87 -> 116 us), but for up to 32 channels per warp (94 x 58 x 5, C = 32: 16.5 -> 13.4 us).
 // Row tiles of 32 rows without lists 37 and 116 us; fp32 FMAs instead of fragments 48 and 88 us (row quads) or slower.
 
 constexpr int kBwdRows = 16;       // texel rows of a warp's tile
@@ -146,10 +147,11 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// NT: channels per warp / 8.  SUM: the reduce mode without counts of other cameras.  (Every stage is in the kernel once and small:
+// NT: channels per warp / 8.  SUM: the reduce mode without counts of other cameras.  WHOLE: the channels fill the warps' tiles (a quarter
+// of the products' instructions would be checks).  (Every stage is in the kernel once and small:
 // a CTA runs most of it once, through an instruction cache that it shares with others at other stages.)
-template <int NT, bool SUM>
-__global__ void __launch_bounds__(kBwdMaxWarps * 32, 2) vt_texel_backward_kernel(const BwdParams q)
+template <int NT, bool SUM, bool WHOLE>
+__global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_backward_kernel(const BwdParams q)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int list_n, slots_n[kBwdMaxTiles];
@@ -186,15 +188,21 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, 2) vt_texel_backward_kernel
     __syncthreads();
     if (tid < 5) sm.tile[tid] = bwd_condition(p, M, tid, xt - 1, xt + 1, ya - 1, ya + rows);
     if (!SUM) {
-        for (int i = tid; i < p.N * 5; i += threads) {
-            const int m = i / 5, t = i - m * 5;
+        for (int i = tid; i < p.N * 10; i += threads) {
+            const int mt = i < p.N * 5 ? i : i - p.N * 5, m = mt / 5, t = mt - m * 5;
             const double *A = sm.mats + m * 12;
-            sm.sees[i] = bwd_condition(p, A, t, -1, p.Wf, -1, p.Hf);
+            if (i < p.N * 5) {
+                sm.sees[mt] = bwd_condition(p, A, t, -1, p.Wf, -1, p.Hf);
+                continue;
+            }
             // d > 0.1, fx > -1/2, fx < Wf - 1/2 (times the depth), likewise fy
-            const double wf = (double)p.Wf, hf = (double)p.Hf;
-            auto row = [&](int e) { return t == 0 ? A[8 + e] : t == 1 ? A[e] : t == 2 ? wf * A[8 + e] - A[e] : t == 3 ? A[4 + e] : hf * A[8 + e] - A[4 + e]; };
-            double *x = sm.exact[i];
-            x[0] = row(0), x[1] = row(1), x[2] = row(3) + row(2) * zl - (t == 0 ? kDepthMin : 0.0), x[3] = row(2) * p.dz;
+            const double size = t == 2 ? (double)p.Wf : (double)p.Hf;
+            const double *B = A + (t == 0 ? 8 : t <= 2 ? 0 : 4);
+            double u[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) u[e] = t == 2 || t == 4 ? size * A[8 + e] - B[e] : B[e];
+            double *x = sm.exact[mt];
+            x[0] = u[0], x[1] = u[1], x[2] = u[3] + u[2] * zl - (t == 0 ? kDepthMin : 0.0), x[3] = u[2] * p.dz;
         }
     }
     __syncthreads();
@@ -304,7 +312,7 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, 2) vt_texel_backward_kernel
                             for (int m = 0; m < p.N; ++m) {
                                 bool sees = !(eq1 && m == n);
 #pragma unroll
-                                for (int t = 0; t < 5; ++t) {
+                                for (int t = 0; t < 3; ++t) {  // (depth, left, right)
                                     const BwdCond &c = sm.sees[m * 5 + t];
                                     sees &= !(fmaf(c.cx, xf, fmaf(c.cy, yf, c.cell)) < 0.f);
                                 }
@@ -321,7 +329,7 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, 2) vt_texel_backward_kernel
                         const double a1 = fma(M[5], xy.y, fma(M[4], xy.x, M[7]));
                         const double a2 = fma(M[9], xy.y, fma(M[8], xy.x, M[11]));
                         const double wlim = (double)p.Wf - 0.5, hlim = (double)p.Hf - 0.5;
-                        constexpr int K = 4;  // bins projected together: a projection is a chain of a dozen fp64 operations
+                        constexpr int K = NT <= 4 ? 2 : 4;  // bins projected together: a projection is a chain of a dozen fp64 operations
                         for (int k0 = klo; k0 <= khi; k0 += K) {
                             int rr[K];
                             float wx[K], ty[K];
@@ -381,7 +389,7 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, 2) vt_texel_backward_kernel
                         float ga[NT], gb[NT];
 #pragma unroll
                         for (int j = 0; j < NT; ++j) {
-                            const bool in = ch0 + 8 * j + (lane >> 2) < p.C;
+                            const bool in = WHOLE || ch0 + 8 * j + (lane >> 2) < p.C;
                             ga[j] = in ? __ldg(pa + 8 * j) : 0.f, gb[j] = in ? __ldg(pb + 8 * j) : 0.f;
                         }
                         uint32_t ah[4], al[4];
