@@ -48,7 +48,6 @@ struct KParams {
     int out_nchw;               // tiled kernel: scalar stores with the strides below (planar output, or ragged channels-last rows)
     int out_c;                  // ... channels of the output (the kernel's C may be padded)
     size_t out_bs, out_cells, out_chs;  // ... element strides of batch element, cell and channel
-    int pdl;                    // host only: launch the forward with programmatic stream serialization
     int tell_late;              // another kernel of the same call follows: start it only after the wait for what ran before
     int accumulate;             // add the result to the fp32 output instead of overwriting it (multi-resolution levels)
     double sx, sy;              // image px -> feature px
@@ -454,6 +453,8 @@ __global__ void __launch_bounds__(128, V == 1 && BF16 ? 7 : (V <= 2 ? 5 : 3)) sc
         const int h = hl / p.L, l = hl - h * p.L;
         dec[i] = ((uint32_t)h << 24) | ((uint32_t)l << 16) | ((uint32_t)(j % p.Zref) << 8) | (uint32_t)j;
     }
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // (nothing of the kernel before has been read)
     __syncthreads();
 
     const unsigned Q = (unsigned)(p.X * p.Y);
@@ -923,6 +924,21 @@ bool padded_tiled_applicable(const flashbev_vt_params *p)
     return need && p->workspace_bytes >= need && (uintptr_t)p->workspace % 16 == 0;
 }
 
+int use_pdl() { return getenv("FLASHBEV_NO_PDL") ? 0 : 1; }
+
+// A kernel whose CTAs may be placed while the kernel before it in the stream drains; it waits for that one's end itself.
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const A &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid, cfg.blockDim = block, cfg.dynamicSmemBytes = smem, cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    if (use_pdl()) cfg.attrs = attr, cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <int V, bool BF16, int WARPS, bool BWD, bool WIDE = false, bool PLANAR = false>
 cudaError_t launch_tiled_inst(const KParams &k, dim3 grid, size_t smem, cudaStream_t stream)
 {
@@ -931,17 +947,9 @@ cudaError_t launch_tiled_inst(const KParams &k, dim3 grid, size_t smem, cudaStre
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    if (!BWD && k.pdl) {
-        // forward launches may overlap their start with the end of the kernel before them in the stream (the kernel
-        // waits for that kernel's completion before it reads or writes global memory)
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = grid, cfg.blockDim = dim3(WARPS * 32), cfg.dynamicSmemBytes = smem, cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr, cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, vt_tiled_kernel<V, BF16, WARPS, BWD, WIDE, PLANAR>, k);
-    }
+    // forward launches may overlap their start with the end of the kernel before them in the stream (the kernel
+    // waits for that kernel's completion before it reads or writes global memory)
+    if (!BWD) return launch_dependent(vt_tiled_kernel<V, BF16, WARPS, BWD, WIDE, PLANAR>, grid, dim3(WARPS * 32), smem, stream, k);
     vt_tiled_kernel<V, BF16, WARPS, BWD, WIDE, PLANAR><<<grid, dim3(WARPS * 32), smem, stream>>>(k);
     return cudaSuccess;
 }
@@ -962,8 +970,6 @@ cudaError_t launch_tiled_warps(int warps, const KParams &k, dim3 grid, size_t sm
             return launch_tiled_inst<V, BF16, 4, false>(k, grid, smem, stream);
     }
 }
-
-int use_pdl() { return getenv("FLASHBEV_NO_PDL") ? 0 : 1; }
 
 // Chooses the channel mapping, super-block shape, run length, list size and grid of the tiled kernel.
 flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V, int &warps, dim3 &grid, size_t &smem,
@@ -1123,7 +1129,6 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
         if (scalar_out == 1) k.out_c = out_c, k.out_bs = plane * out_c, k.out_cells = 1, k.out_chs = plane;
         if (scalar_out == 2) k.out_c = out_c, k.out_bs = plane * out_c, k.out_cells = out_c, k.out_chs = 1;
     }
-    k.pdl = use_pdl();
     k.tell_late = tell_late;
     const bool bf16 = p->feat_dtype == FLASHBEV_BF16;
     cudaError_t e;
@@ -1179,8 +1184,7 @@ cudaError_t launch_backward(const BwdParams &q, dim3 grid, size_t smem, cudaStre
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    kernel<<<grid, dim3((unsigned)(q.row_tiles * q.ch_tiles * q.groups * 32)), smem, stream>>>(q);
-    return cudaSuccess;
+    return launch_dependent(kernel, grid, dim3((unsigned)(q.row_tiles * q.ch_tiles * q.groups * 32)), smem, stream, q);
 }
 
 // Which of the two backward kernels takes a call: the texel-side one, but not
@@ -1228,19 +1232,6 @@ flashbev_status launch_texel_backward(const flashbev_vt_params *p, const float *
     return FLASHBEV_OK;
 }
 
-// A copy kernel (256 threads), which waits for the kernel before it in the stream and then lets the tiled kernel start.
-template <typename... P, typename... A>
-void launch_copy(void (*kernel)(P...), dim3 grid, cudaStream_t stream, A... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid, cfg.blockDim = dim3(256), cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    if (use_pdl()) cfg.attrs = attr, cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
-}
-
 // NCHW tensors on the tiled kernel: features -> channels-last copy in the workspace, output written planar.
 flashbev_status launch_nchw_tiled(const flashbev_vt_params *p, cudaStream_t stream, bool accumulate)
 {
@@ -1263,7 +1254,7 @@ flashbev_status launch_nchw_tiled(const flashbev_vt_params *p, cudaStream_t stre
     const dim3 grid((unsigned)((HW + 64 * E - 1) / (64 * E)), (unsigned)((q.C + 4 * E - 1) / (4 * E)), (unsigned)(p->B * p->N));
     auto copy = [&](auto kernel, auto *elem) {
         using T = typename std::remove_pointer<decltype(elem)>::type;
-        launch_copy(kernel, grid, stream, static_cast<const T *>(p->features), static_cast<T *>(p->workspace), p->C, q.C, HW);
+        launch_dependent(kernel, grid, dim3(256), 0, stream, static_cast<const T *>(p->features), static_cast<T *>(p->workspace), p->C, q.C, HW);
     };
     if (E == 8 && aligned) copy(nchw_to_nhwc_kernel<uint16_t, true>, (uint16_t *)nullptr);
     else if (E == 8) copy(nchw_to_nhwc_kernel<uint16_t, false>, (uint16_t *)nullptr);
@@ -1295,10 +1286,10 @@ flashbev_status launch_padded_tiled(const flashbev_vt_params *p, cudaStream_t st
     const unsigned total = (unsigned)p->N * p->feat_h * p->feat_w * vecs;  // < 2^31 (pad_copy_bytes)
     const dim3 blocks((total + 255) / 256, (unsigned)p->B);
     if (p->feat_dtype == FLASHBEV_BF16)
-        launch_copy(pad_channels_kernel<uint16_t>, blocks, stream, static_cast<const uint16_t *>(p->features),
+        launch_dependent(pad_channels_kernel<uint16_t>, blocks, dim3(256), 0, stream, static_cast<const uint16_t *>(p->features),
                     static_cast<uint4 *>(p->workspace), total, p->C, (unsigned)vecs);
     else
-        launch_copy(pad_channels_kernel<float>, blocks, stream, static_cast<const float *>(p->features),
+        launch_dependent(pad_channels_kernel<float>, blocks, dim3(256), 0, stream, static_cast<const float *>(p->features),
                     static_cast<uint4 *>(p->workspace), total, p->C, (unsigned)vecs);
     if (cudaGetLastError() != cudaSuccess) return FLASHBEV_CUDA_ERROR;
     const flashbev_status st = launch_tiled(&q, stream, accumulate, false, 2, p->C);
@@ -1583,8 +1574,7 @@ flashbev_status flashbev_sca(const flashbev_sca_params *q, void *stream_)
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kern<<<dim3((unsigned)blocks), dim3(128), smem, stream>>>(k);
-        return cudaSuccess;
+        return launch_dependent(kern, dim3((unsigned)blocks), dim3(128), smem, stream, k);
     };
     cudaError_t e;
     const bool even = k.hp * k.lph == 32 && q->heads == V * k.hp;

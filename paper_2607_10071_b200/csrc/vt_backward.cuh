@@ -163,6 +163,10 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_b
     BwdSmem sm;
     bwd_smem_layout(smem_raw, &sm, p.N, q.row_tiles, q.ch_tiles, q.groups, NT, p.reduce);
 
+    // (programmatic dependent launch: this grid's CTAs are placed while the one before drains, as in the forward)
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
     // ---- which texel column (rows from blockIdx.z on, channels from blockIdx.y on)
     const unsigned column = blockIdx.x / (unsigned)q.slices, slice = blockIdx.x - column * (unsigned)q.slices;
     const unsigned cam = column / (unsigned)p.Wf;
