@@ -48,7 +48,7 @@ struct KParams {
     int out_nchw;               // tiled kernel: scalar stores with the strides below (planar output, or ragged channels-last rows)
     int out_c;                  // ... channels of the output (the kernel's C may be padded)
     size_t out_bs, out_cells, out_chs;  // ... element strides of batch element, cell and channel
-    int tell_late;              // another kernel of the same call follows: start it only after the wait for what ran before
+    int level;                  // 1: the first level of a pyramid, 2: a later one, 0: not of one
     int accumulate;             // add the result to the fp32 output instead of overwriting it (multi-resolution levels)
     double sx, sy;              // image px -> feature px
     double x_min, dx, y_min, dy, z_min, dz;
@@ -939,18 +939,18 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
-template <int V, bool BF16, int WARPS, bool BWD, bool WIDE = false, bool PLANAR = false>
+template <int V, bool BF16, int WARPS, bool BWD, bool WIDE = false, bool PLANAR = false, bool LEVEL = false>
 cudaError_t launch_tiled_inst(const KParams &k, dim3 grid, size_t smem, cudaStream_t stream)
 {
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(vt_tiled_kernel<V, BF16, WARPS, BWD, WIDE, PLANAR>,
+        cudaError_t e = cudaFuncSetAttribute(vt_tiled_kernel<V, BF16, WARPS, BWD, WIDE, PLANAR, LEVEL>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     // forward launches may overlap their start with the end of the kernel before them in the stream (the kernel
     // waits for that kernel's completion before it reads or writes global memory)
-    if (!BWD) return launch_dependent(vt_tiled_kernel<V, BF16, WARPS, BWD, WIDE, PLANAR>, grid, dim3(WARPS * 32), smem, stream, k);
-    vt_tiled_kernel<V, BF16, WARPS, BWD, WIDE, PLANAR><<<grid, dim3(WARPS * 32), smem, stream>>>(k);
+    if (!BWD) return launch_dependent(vt_tiled_kernel<V, BF16, WARPS, BWD, WIDE, PLANAR, LEVEL>, grid, dim3(WARPS * 32), smem, stream, k);
+    vt_tiled_kernel<V, BF16, WARPS, BWD, WIDE, PLANAR, LEVEL><<<grid, dim3(WARPS * 32), smem, stream>>>(k);
     return cudaSuccess;
 }
 
@@ -965,6 +965,10 @@ cudaError_t launch_tiled_warps(int warps, const KParams &k, dim3 grid, size_t sm
             if (k.out_nchw) {  // (planar output: instances for 4 warps per CTA only)
                 if (V % 2 == 0 && k.wide) return launch_tiled_inst<V, BF16, 4, false, (V % 2 == 0), true>(k, grid, smem, stream);
                 return launch_tiled_inst<V, BF16, 4, false, false, true>(k, grid, smem, stream);
+            }
+            if (k.level && (V > 1 || BF16)) {  // (instances for 4 warps per CTA only)
+                if (V % 2 == 0 && k.wide) return launch_tiled_inst<V, BF16, 4, false, (V % 2 == 0), false, true>(k, grid, smem, stream);
+                return launch_tiled_inst<V, BF16, 4, false, false, false, true>(k, grid, smem, stream);
             }
             if (V % 2 == 0 && k.wide) return launch_tiled_inst<V, BF16, 4, false, (V % 2 == 0)>(k, grid, smem, stream);
             return launch_tiled_inst<V, BF16, 4, false>(k, grid, smem, stream);
@@ -1114,14 +1118,16 @@ flashbev_status configure_tiled(const flashbev_vt_params *p, KParams &k, int &V,
 
 // scalar_out: 0 vector stores into channels-last rows; 1 planar output [B][out_c][X][Y]; 2 channels-last rows of out_c
 // channels (the kernel's own C may be padded)
-flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, bool accumulate = false, bool tell_late = false,
+flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, bool accumulate = false, bool pyramid = false,
                              int scalar_out = 0, int out_c = 0)
 {
     KParams k;
     int V, warps;
     dim3 grid;
     size_t smem;
-    const flashbev_status st = configure_tiled(p, k, V, warps, grid, smem, accumulate, false, scalar_out == 1);
+    flashbev_vt_params q = *p;
+    if (pyramid) q.tune[3] = (q.tune[3] & ~0xf) | 4;  // the instances for pyramid levels are built for 4 warps per CTA
+    const flashbev_status st = configure_tiled(&q, k, V, warps, grid, smem, accumulate, false, scalar_out == 1);
     if (st != FLASHBEV_OK) return st;
     k.out_nchw = scalar_out != 0;
     {
@@ -1129,7 +1135,7 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
         if (scalar_out == 1) k.out_c = out_c, k.out_bs = plane * out_c, k.out_cells = 1, k.out_chs = plane;
         if (scalar_out == 2) k.out_c = out_c, k.out_bs = plane * out_c, k.out_cells = out_c, k.out_chs = 1;
     }
-    k.tell_late = tell_late;
+    k.level = pyramid ? (accumulate ? 2 : 1) : 0;
     const bool bf16 = p->feat_dtype == FLASHBEV_BF16;
     cudaError_t e;
     static const char *const names[2][4] = {{"tiled_f32_v1", "tiled_f32_v2", "tiled_f32_v3", "tiled_f32_v4"},
@@ -1148,16 +1154,21 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
     return e == cudaSuccess ? FLASHBEV_OK : FLASHBEV_CUDA_ERROR;
 }
 
-// Chooses the tiles and the grid of the texel-side backward kernel.  NT: channels per warp / 8.
-flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, int &NT, dim3 &grid, size_t &smem)
+// Chooses the tiles and the grid of the texel-side backward kernel.  NT: channels per warp / 8; RT: row tiles per warp.
+flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, int &NT, int &RT, dim3 &grid, size_t &smem)
 {
     q = {};
     q.k = base_params(p);
-    const int ch_tiles = (p->C + 79) / 80;
-    NT = ((p->C + ch_tiles - 1) / ch_tiles + 15) / 16 * 2;  // (instances for every other NT)
     q.row_tiles = std::min(kBwdMaxTiles, (p->feat_h + kBwdRows - 1) / kBwdRows);
-    q.ch_tiles = std::min(ch_tiles, kBwdMaxWarps / q.row_tiles);
-    q.groups = std::max(1, 4 / (q.row_tiles * q.ch_tiles));
+    // Three or four row tiles: the middle ones, about the horizon, have most of the cells, so a warp takes two of them, a long and a
+    // short one, and half the channels (us, one / two row tiles per warp: 56 x 100 maps, C = 128, tilted 85.9 / 79.3; 51 x 40, C = 128
+    // 63.0 / 57.1; 38 x 56, C = 80 105 / 77; 48 x 162, C = 80, tilted 62.4 / 62.5; 48 channels per warp 96, 65, 84, 63).
+    RT = q.row_tiles > 2 && p->C <= 128 ? 2 : 1;
+    q.row_warps = (q.row_tiles + RT - 1) / RT;
+    const int most = RT == 2 ? 32 : 80, ch_tiles = (p->C + most - 1) / most;
+    NT = ((p->C + ch_tiles - 1) / ch_tiles + 15) / 16 * 2;  // (instances for every other NT)
+    q.ch_tiles = std::min(ch_tiles, kBwdMaxWarps / q.row_warps);
+    q.groups = std::max(1, 4 / (q.row_warps * q.ch_tiles));
     const int rows = q.row_tiles * kBwdRows, channels = 8 * NT * q.ch_tiles;
     const int cblocks = (p->C + channels - 1) / channels, rblocks = (p->feat_h + rows - 1) / rows;
     const double columns = (double)p->B * p->N * p->feat_w * cblocks * rblocks;
@@ -1167,24 +1178,24 @@ flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, in
     // 528, 40 k, C = 80 33 / 37 / 39.
     q.slices = columns <= 2.0 * sm_count() && (double)p->X * p->Y > 100.0 * p->N * p->feat_w ? 2 : 1;
     q.exclusive = q.slices == 1;
-    smem = bwd_smem_layout(nullptr, nullptr, p->N, q.row_tiles, q.ch_tiles, q.groups, NT, p->reduce);
+    smem = bwd_smem_layout(nullptr, nullptr, p->N, q.row_tiles, q.row_warps, q.ch_tiles, q.groups, NT, RT, p->reduce);
     const double blocks = (double)p->B * p->N * p->feat_w * q.slices;
     if (blocks > 2147483647.0 || cblocks > 65535 || rblocks > 65535 || smem > 200 * 1024) return FLASHBEV_UNSUPPORTED;
     grid = dim3((unsigned)blocks, (unsigned)cblocks, (unsigned)rblocks);
     return FLASHBEV_OK;
 }
 
-template <int NT>
+template <int NT, int RT = 1>
 cudaError_t launch_backward(const BwdParams &q, dim3 grid, size_t smem, cudaStream_t stream)
 {
     const bool sum = q.k.reduce == FLASHBEV_REDUCE_SUM, full = q.k.C == (int)grid.y * q.ch_tiles * 8 * NT;
-    const auto kernel = sum ? (full ? vt_texel_backward_kernel<NT, true, true> : vt_texel_backward_kernel<NT, true, false>)
-                            : (full ? vt_texel_backward_kernel<NT, false, true> : vt_texel_backward_kernel<NT, false, false>);
+    const auto kernel = sum ? (full ? vt_texel_backward_kernel<NT, RT, true, true> : vt_texel_backward_kernel<NT, RT, true, false>)
+                            : (full ? vt_texel_backward_kernel<NT, RT, false, true> : vt_texel_backward_kernel<NT, RT, false, false>);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    return launch_dependent(kernel, grid, dim3((unsigned)(q.row_tiles * q.ch_tiles * q.groups * 32)), smem, stream, q);
+    return launch_dependent(kernel, grid, dim3((unsigned)(q.row_warps * q.ch_tiles * q.groups * 32)), smem, stream, q);
 }
 
 // Which of the two backward kernels takes a call: the texel-side one, but not
@@ -1206,10 +1217,10 @@ bool backward_by_texel(const flashbev_vt_params *p)
 flashbev_status launch_texel_backward(const flashbev_vt_params *p, const float *grad_out, float *grad_features, cudaStream_t stream)
 {
     BwdParams q;
-    int NT;
+    int NT, RT;
     dim3 grid;
     size_t smem;
-    const flashbev_status st = configure_backward(p, q, NT, grid, smem);
+    const flashbev_status st = configure_backward(p, q, NT, RT, grid, smem);
     if (st != FLASHBEV_OK) return st;
     q.k.feat = nullptr, q.k.out = nullptr, q.k.count_out = nullptr;
     q.k.gout = grad_out, q.k.gfeat = grad_features;
@@ -1221,7 +1232,9 @@ flashbev_status launch_texel_backward(const flashbev_vt_params *p, const float *
         }
     }
     cudaError_t e;
-    if (NT <= 2) e = launch_backward<2>(q, grid, smem, stream);
+    if (RT == 2 && NT <= 2) e = launch_backward<2, 2>(q, grid, smem, stream);
+    else if (RT == 2) e = launch_backward<4, 2>(q, grid, smem, stream);
+    else if (NT <= 2) e = launch_backward<2>(q, grid, smem, stream);
     else if (NT <= 4) e = launch_backward<4>(q, grid, smem, stream);
     else if (NT <= 6) e = launch_backward<6>(q, grid, smem, stream);
     else if (NT <= 8) e = launch_backward<8>(q, grid, smem, stream);
@@ -1330,7 +1343,7 @@ flashbev_status run_device(const flashbev_vt_params *p, cudaStream_t stream, int
     }
     const bool tiled = p->kernel == FLASHBEV_KERNEL_TILED || (p->kernel == FLASHBEV_KERNEL_AUTO && tiled_applicable(p));
     if (tiled && !tiled_applicable(p)) return FLASHBEV_UNSUPPORTED;
-    st = tiled ? launch_tiled(p, stream, accumulate, level == 0 && levels > 1) : launch_per_output(p, stream, accumulate);
+    st = tiled ? launch_tiled(p, stream, accumulate, levels > 1) : launch_per_output(p, stream, accumulate);
     // AUTO: shapes the tiled kernel cannot be configured for (nothing was launched) go to the generic kernel
     if (tiled && st == FLASHBEV_UNSUPPORTED && p->kernel == FLASHBEV_KERNEL_AUTO) st = launch_per_output(p, stream, accumulate);
     if (st != FLASHBEV_OK) return st;

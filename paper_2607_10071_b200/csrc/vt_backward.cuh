@@ -22,7 +22,7 @@
 //
 // Why: the scatter hands two fp32 vector reductions per record to the crossbar -- 11.5 M sectors for a gradient of 0.17 M on
 // 200 x 200 x 8, C = 80 -- and is bound by the rate at which an SM can do that (92 us).  Here a texel leaves the SM once: 33 us;
-// 56 x 100 maps of tilted cameras, C = 128, Eq. 1: 144 -> 87 us.  What bounds it now: no unit (issue 34 %, tensor pipe 17 %); 16
+// 56 x 100 maps of tilted cameras, C = 128, Eq. 1: 144 -> 79 us.  What bounds it now: no unit (issue 34 %, tensor pipe 17 %); 16
 // warps per SM that wait at the barriers of a round, for grad_out and for chains of fp64 operations, in 0.9 to 2 waves of CTAs of
 // unequal size.  128 registers: with 80 (24 warps per SM) the spills cost more than the warps bring
 // (calibrated 87 -> 116 us), but for up to 32 channels per warp (94 x 58 x 5, C = 32: 16.5 -> 13.4 us).
@@ -36,7 +36,8 @@ constexpr int kBwdDeal = 8;        // cells along y that go to the same slice
 
 struct BwdParams {
     KParams k;
-    int row_tiles, ch_tiles, groups;  // warps of a CTA: groups of row_tiles x ch_tiles tiles
+    int row_tiles;                    // tiles of 16 rows per CTA
+    int row_warps, ch_tiles, groups;  // warps of a CTA: groups of row_warps x ch_tiles; a warp has every row_warps-th row tile
     int slices;                       // CTAs that share a texel column, each with its share of the cells
     int first_map;                    // the first b * N + n of the launch
     int exclusive;                    // one CTA per column: results are stored, not added
@@ -60,8 +61,8 @@ struct BwdSmem {
     uint8_t *slots;        // [row_tiles][32 warps]: the round's cells that have weights in the row tile
 };
 
-__host__ __device__ inline size_t bwd_smem_layout(unsigned char *base, BwdSmem *t, int N, int row_tiles, int ch_tiles, int groups, int NT,
-                                                  int reduce)
+__host__ __device__ inline size_t bwd_smem_layout(unsigned char *base, BwdSmem *t, int N, int row_tiles, int row_warps, int ch_tiles, int groups,
+                                                  int NT, int RT, int reduce)
 {
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -69,9 +70,9 @@ __host__ __device__ inline size_t bwd_smem_layout(unsigned char *base, BwdSmem *
         o += align16(bytes);
         return ptr;
     };
-    const size_t warps = (size_t)row_tiles * ch_tiles * groups, all = reduce == FLASHBEV_REDUCE_SUM ? 0 : (size_t)N;
+    const size_t warps = (size_t)row_warps * ch_tiles * groups, all = reduce == FLASHBEV_REDUCE_SUM ? 0 : (size_t)N;
     const size_t weights = (size_t)row_tiles * kBwdRows * (32 * warps + 4) * sizeof(float);
-    const size_t sums = (size_t)(groups - 1) * row_tiles * ch_tiles * NT * 32 * sizeof(float4);
+    const size_t sums = (size_t)(groups - 1) * row_warps * ch_tiles * RT * NT * 32 * sizeof(float4);
     unsigned char *p0 = take(weights > sums ? weights : sums);
     unsigned char *p1 = take((all ? all : 1) * 12 * sizeof(double));
     unsigned char *p2 = take(all * 5 * 4 * sizeof(double));
@@ -147,11 +148,11 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// NT: channels per warp / 8.  SUM: the reduce mode without counts of other cameras.  WHOLE: the channels fill the warps' tiles (a quarter
+// NT: channels per warp / 8.  RT: row tiles per warp.  SUM: the reduce mode without counts of other cameras.  WHOLE: the channels fill the warps' tiles (a quarter
 // of the products' instructions would be checks).  (Every stage is in the kernel once and small:
 // a CTA runs most of it once, through an instruction cache that it shares with others at other stages.)
-template <int NT, bool SUM, bool WHOLE>
-__global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_backward_kernel(const BwdParams q)
+template <int NT, int RT, bool SUM, bool WHOLE>
+__global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_texel_backward_kernel(const BwdParams q)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int list_n, slots_n[kBwdMaxTiles];
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_b
     const unsigned lt_mask = (1u << lane) - 1u;
     const bool eq1 = !SUM && p.reduce == FLASHBEV_REDUCE_CAMERA_MEAN_Z_SUM;
     BwdSmem sm;
-    bwd_smem_layout(smem_raw, &sm, p.N, q.row_tiles, q.ch_tiles, q.groups, NT, p.reduce);
+    bwd_smem_layout(smem_raw, &sm, p.N, q.row_tiles, q.row_warps, q.ch_tiles, q.groups, NT, RT, p.reduce);
 
     // (programmatic dependent launch: this grid's CTAs are placed while the one before drains, as in the forward)
     asm volatile("griddepcontrol.launch_dependents;");
@@ -211,14 +212,16 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_b
     }
     __syncthreads();
 
-    // ---- role of the warp in the products: rows [16 row_tile, ..), channels [ch0, ch0 + 8 NT)
-    const int tiles = q.row_tiles * q.ch_tiles, group = warp / tiles, row_tile = (warp - group * tiles) / q.ch_tiles;
+    // ---- role of the warp in the products: row tiles row_warp, + row_warps, channels [ch0, ch0 + 8 NT)
+    const int tiles = q.row_warps * q.ch_tiles, group = warp / tiles, row_warp = (warp - group * tiles) / q.ch_tiles;
     const int ch0 = (blockIdx.y * q.ch_tiles + warp % q.ch_tiles) * (NT * 8);
-    float2 acc[NT][2];  // fragment layout: rows lane / 4 and + 8, channels 2 (lane % 4) and + 1
+    float2 acc[RT][NT][2];  // fragment layout: rows lane / 4 and + 8, channels 2 (lane % 4) and + 1
     const float *const gout = p.gout + (size_t)b * p.X * p.Y * p.C;
     const float x_first = (float)(p.x_min + 0.5 * p.dx), y_first = (float)(p.y_min + 0.5 * p.dy), dxf = (float)p.dx, dyf = (float)p.dy;
 #pragma unroll
-    for (int j = 0; j < NT; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int j = 0; j < NT; ++j) acc[i][j][0] = acc[i][j][1] = make_float2(0.f, 0.f);
     // (a second pass, if a grad_out that is not finite was met: see the end)
     for (bool again = false;; again = true) {
         int row0 = 32 * (warp - warps);           // a chunk is 32 grid rows, a row per lane
@@ -333,7 +336,7 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_b
                         const double a1 = fma(M[5], xy.y, fma(M[4], xy.x, M[7]));
                         const double a2 = fma(M[9], xy.y, fma(M[8], xy.x, M[11]));
                         const double wlim = (double)p.Wf - 0.5, hlim = (double)p.Hf - 0.5;
-                        constexpr int K = NT <= 4 ? 2 : 4;  // bins projected together: a projection is a chain of a dozen fp64 operations
+                        constexpr int K = NT * RT <= 4 ? 2 : 4;  // bins projected together: a projection is a chain of a dozen fp64 operations
                         for (int k0 = klo; k0 <= khi; k0 += K) {
                             int rr[K];
                             float wx[K], ty[K];
@@ -379,42 +382,48 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_b
                 __syncthreads();
 
                 // ---- products: 8 cells at a time
-                const float *const wt = sm.weights + (row_tile * kBwdRows + (lane >> 2)) * pitch;
                 if (!again) {
-                    const uint8_t *const slots = sm.slots + row_tile * 32 * warps;
-                    const int n_slots = slots_n[row_tile];
+#pragma unroll
+                    for (int i = 0; i < RT; ++i) {
+                        const int row_tile = row_warp + i * q.row_warps;
+                        if (RT > 1 && row_tile >= q.row_tiles) break;
+                        const float *const wt = sm.weights + (row_tile * kBwdRows + (lane >> 2)) * pitch;
+                        const uint8_t *const slots = sm.slots + row_tile * 32 * warps;
+                        const int n_slots = slots_n[row_tile];
 #pragma unroll 1
-                    for (int k = 8 * group; k < n_slots; k += 8 * q.groups) {
-                        // (cells past the last one: the last one, with weight 0)
-                        const int ka = k + (lane & 3), kb = ka + 4;
-                        const int sa = slots[min(ka, n_slots - 1)], sb = slots[min(kb, n_slots - 1)];
-                        const float *const pa = gout + (size_t)FB_IDX(sm.list[first + sa], p.X * p.Y, p.err) * (unsigned)p.C + ch0 + (lane >> 2);
-                        const float *const pb = gout + (size_t)FB_IDX(sm.list[first + sb], p.X * p.Y, p.err) * (unsigned)p.C + ch0 + (lane >> 2);
-                        float ga[NT], gb[NT];
+                        for (int k = 8 * group; k < n_slots; k += 8 * q.groups) {
+                            // (cells past the last one: the last one, with weight 0)
+                            const int ka = k + (lane & 3), kb = ka + 4;
+                            const int sa = slots[min(ka, n_slots - 1)], sb = slots[min(kb, n_slots - 1)];
+                            const float *const pa = gout + (size_t)FB_IDX(sm.list[first + sa], p.X * p.Y, p.err) * (unsigned)p.C + ch0 + (lane >> 2);
+                            const float *const pb = gout + (size_t)FB_IDX(sm.list[first + sb], p.X * p.Y, p.err) * (unsigned)p.C + ch0 + (lane >> 2);
+                            float ga[NT], gb[NT];
 #pragma unroll
-                        for (int j = 0; j < NT; ++j) {
-                            const bool in = WHOLE || ch0 + 8 * j + (lane >> 2) < p.C;
-                            ga[j] = in ? __ldg(pa + 8 * j) : 0.f, gb[j] = in ? __ldg(pb + 8 * j) : 0.f;
-                        }
-                        uint32_t ah[4], al[4];
-                        split_tf32(ka < n_slots ? wt[sa] : 0.f, ah[0], al[0]), split_tf32(ka < n_slots ? wt[8 * pitch + sa] : 0.f, ah[1], al[1]);
-                        split_tf32(kb < n_slots ? wt[sb] : 0.f, ah[2], al[2]), split_tf32(kb < n_slots ? wt[8 * pitch + sb] : 0.f, ah[3], al[3]);
+                            for (int j = 0; j < NT; ++j) {
+                                const bool in = WHOLE || ch0 + 8 * j + (lane >> 2) < p.C;
+                                ga[j] = in ? __ldg(pa + 8 * j) : 0.f, gb[j] = in ? __ldg(pb + 8 * j) : 0.f;
+                            }
+                            uint32_t ah[4], al[4];
+                            split_tf32(ka < n_slots ? wt[sa] : 0.f, ah[0], al[0]), split_tf32(ka < n_slots ? wt[8 * pitch + sa] : 0.f, ah[1], al[1]);
+                            split_tf32(kb < n_slots ? wt[sb] : 0.f, ah[2], al[2]), split_tf32(kb < n_slots ? wt[8 * pitch + sb] : 0.f, ah[3], al[3]);
 #pragma unroll
-                        for (int j = 0; j < NT; ++j) {
-                            uint32_t bh[2], bl[2];
-                            split_tf32(ga[j], bh[0], bl[0]), split_tf32(gb[j], bh[1], bl[1]);
-                            float t[4] = {0.f, 0.f, 0.f, 0.f};
-                            mma_tf32(t, al, bh[0], bh[1]);
-                            mma_tf32(t, ah, bl[0], bl[1]);
-                            mma_tf32(t, ah, bh[0], bh[1]);
-                            acc[j][0] = __fadd2_rn(acc[j][0], make_float2(t[0], t[1]));
-                            acc[j][1] = __fadd2_rn(acc[j][1], make_float2(t[2], t[3]));
+                            for (int j = 0; j < NT; ++j) {
+                                uint32_t bh[2], bl[2];
+                                split_tf32(ga[j], bh[0], bl[0]), split_tf32(gb[j], bh[1], bl[1]);
+                                float t[4] = {0.f, 0.f, 0.f, 0.f};
+                                mma_tf32(t, al, bh[0], bh[1]);
+                                mma_tf32(t, ah, bl[0], bl[1]);
+                                mma_tf32(t, ah, bh[0], bh[1]);
+                                acc[i][j][0] = __fadd2_rn(acc[i][j][0], make_float2(t[0], t[1]));
+                                acc[i][j][1] = __fadd2_rn(acc[i][j][1], make_float2(t[2], t[3]));
+                            }
                         }
                     }
                 } else if (group == 0) {
                     for (int c = 0; c < min(32 * warps, waiting - first); ++c) {
                         const float *src = gout + (size_t)FB_IDX(sm.list[first + c], p.X * p.Y, p.err) * (unsigned)p.C;
-                        for (int r = row_tile * kBwdRows; r < min((row_tile + 1) * kBwdRows, rv); ++r) {
+                        for (int r = row_warp * kBwdRows; r < rv; ++r) {
+                            if (r / kBwdRows % q.row_warps != row_warp) continue;
                             const float w = sm.weights[r * pitch + c];
                             if (w == 0.f) continue;
                             for (int ch = ch0 + lane; ch < min(ch0 + 8 * NT, p.C); ch += 32) atomicAdd(dst + (size_t)r * rowf + ch, w * __ldg(src + ch));
@@ -435,9 +444,11 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_b
         // stays zero for now and is made once more, record by record.
         float big = 0.f;
 #pragma unroll
-        for (int j = 0; j < NT; ++j)
+        for (int i = 0; i < RT; ++i)
 #pragma unroll
-            for (int h = 0; h < 2; ++h) big = fmaf(acc[j][h].x, 0.f, big), big = fmaf(acc[j][h].y, 0.f, big);
+            for (int j = 0; j < NT; ++j)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) big = fmaf(acc[i][j][h].x, 0.f, big), big = fmaf(acc[i][j][h].y, 0.f, big);
         const bool odd = __syncthreads_or(big != 0.f);
 
         // ---- the groups' sums, then the column's gradient leaves the SM
@@ -445,24 +456,29 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_b
             float4 *const sums = reinterpret_cast<float4 *>(sm.weights) + lane;
             if (group > 0) {
 #pragma unroll
-                for (int j = 0; j < NT; ++j)
-                    sums[((warp - tiles) * NT + j) * 32] = make_float4(acc[j][0].x, acc[j][0].y, acc[j][1].x, acc[j][1].y);
+                for (int i = 0; i < RT; ++i)
+#pragma unroll
+                    for (int j = 0; j < NT; ++j)
+                        sums[(((warp - tiles) * RT + i) * NT + j) * 32] =
+                            make_float4(acc[i][j][0].x, acc[i][j][0].y, acc[i][j][1].x, acc[i][j][1].y);
             }
             __syncthreads();
             if (group == 0)
 #pragma unroll 1
                 for (int g = 1; g < q.groups; ++g)
 #pragma unroll
-                    for (int j = 0; j < NT; ++j) {
-                        const float4 v = sums[((warp + (g - 1) * tiles) * NT + j) * 32];
-                        acc[j][0] = __fadd2_rn(acc[j][0], make_float2(v.x, v.y));
-                        acc[j][1] = __fadd2_rn(acc[j][1], make_float2(v.z, v.w));
-                    }
+                    for (int i = 0; i < RT; ++i)
+#pragma unroll
+                        for (int j = 0; j < NT; ++j) {
+                            const float4 v = sums[(((warp + (g - 1) * tiles) * RT + i) * NT + j) * 32];
+                            acc[i][j][0] = __fadd2_rn(acc[i][j][0], make_float2(v.x, v.y));
+                            acc[i][j][1] = __fadd2_rn(acc[i][j][1], make_float2(v.z, v.w));
+                        }
         }
         if (group == 0) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = row_tile * kBwdRows + 8 * h + (lane >> 2);
+            for (int ih = 0; ih < 2 * RT; ++ih) {
+                const int i = ih >> 1, h = ih & 1, r = (row_warp + i * q.row_warps) * kBwdRows + 8 * h + (lane >> 2);
                 if (r >= rv) continue;
                 float *row = dst + (size_t)r * rowf + ch0 + 2 * (lane & 3);
 #ifdef FLASHBEV_DEBUG_BOUNDS
@@ -471,7 +487,7 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT <= 4 ? 3 : 2) vt_texel_b
 #pragma unroll
                 for (int j = 0; j < NT; ++j) {
                     if (ch0 + 8 * j + 2 * (lane & 3) >= p.C) continue;  // (C is a multiple of 4)
-                    const float2 v = odd ? make_float2(0.f, 0.f) : acc[j][h];
+                    const float2 v = odd ? make_float2(0.f, 0.f) : acc[i][j][h];
                     if (q.exclusive) *reinterpret_cast<float2 *>(row + 8 * j) = v;
                     else if (v.x != 0.f || v.y != 0.f) atomicAdd(reinterpret_cast<float2 *>(row + 8 * j), v);
                 }

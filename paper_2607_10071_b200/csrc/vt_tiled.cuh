@@ -777,7 +777,8 @@ __device__ __forceinline__ void walk_one(const KParams &p, const WarpSmem &sm, i
 // PLANAR: the output is written one channel at a time with the strides in the parameters -- [B][C][X][Y] tensors, or
 // channels-last rows that are not whole 16-byte vectors (the features are then a copy in the kernel's own layout);
 // instances of their own, so that the vector-store instances do not carry the scalar stores
-template <int V, bool BF16, int WARPS, bool BWD, bool WIDE, bool PLANAR = false>
+// LEVEL: a level of a pyramid; those after the first add to the output (p.accumulate)
+template <int V, bool BF16, int WARPS, bool BWD, bool WIDE, bool PLANAR = false, bool LEVEL = false>
 __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / WARPS)
     vt_tiled_kernel(const KParams p)
 {
@@ -802,12 +803,16 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
     // dependent of the grid before) touch no global memory that the grid before writes until that grid has completed and its
     // writes are visible.  Normally that is any memory, and this is where the wait is.  After a grid of the same call the matrices
     // are nobody's output, and the wait comes later: before the features that a copy made (PLANAR), or before the sum of the
-    // pyramid levels before (accumulate).  Such a grid before lets this one start only when its own wait is over (tell_late),
-    // so that whatever ran before the call has completed.  All are no-ops for a launch without the attribute.
-    // (pyramid of three 105 -> 97 us, planar 74 -> 72 us, ragged rows 48 -> 44 us: a grid's geometry runs in the tail of the one before)
-    const bool chained = !BWD && (PLANAR || p.accumulate);
+    // pyramid levels before (LEVEL).  The copy, or the first level, lets this grid start only when its own wait is over, so that
+    // whatever ran before the call has completed.  All are no-ops for a launch without the attribute.
+    // (pyramid of three 105 -> 96 us, planar 75 -> 71 us, ragged rows 47 -> 44 us: a grid's geometry runs in the tail of the one before.
+    // Instances of their own for pyramid levels take 0.5-1 % off the others, but not of one fp32 vector per lane: there the smallest
+    // calls measure 7.1 us with one instance for both, decided by the parameters, and 7.4 us with two.)
+    constexpr bool kBoth = V == 1 && !BF16 && !PLANAR && !BWD;
+    const bool adds = kBoth ? p.accumulate != 0 : LEVEL && p.accumulate;
+    const bool chained = !BWD && (PLANAR || (kBoth ? adds : LEVEL));
     if (!BWD) {
-        if (p.tell_late) asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (kBoth ? p.level == 1 : LEVEL && !adds) asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;");
         if (!chained) asm volatile("griddepcontrol.wait;" ::: "memory");
     }
@@ -1038,7 +1043,7 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                                     }
                                 }
                             }
-                    } else if (!(p.accumulate | p.out_bf16)) {
+                    } else if (kBoth ? !(p.accumulate | p.out_bf16) : !LEVEL && !p.out_bf16) {
 #pragma unroll
                         for (int v = 0; v < V; ++v)
                             if (von[v]) {
@@ -1055,7 +1060,7 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
                                 for (int e = 0; e < PV; e += 2) {
                                     float4 *dst = reinterpret_cast<float4 *>(o + v * vstride + e * 2);
                                     float4 val = make_float4(acc[v][e].x, acc[v][e].y, acc[v][e + 1].x, acc[v][e + 1].y);
-                                    if (p.accumulate) {  // multi-resolution levels after the first: `dst` holds the other levels' sum
+                                    if (adds) {  // multi-resolution levels after the first: `dst` holds the other levels' sum
                                         asm volatile("griddepcontrol.wait;" ::: "memory");
                                         const float4 prev = __ldcg(dst);
                                         val.x += prev.x, val.y += prev.y, val.z += prev.z, val.w += prev.w;
