@@ -291,7 +291,7 @@ def measure_regimes(torch, df, device):
 
 
 def measure_backward(torch, w, args, device, steps, warmup, dist_barrier):
-    """Latency of flashbev_sampling_vt_backward (memset + scatter kernel) per frame, L2-cold frames."""
+    """Latency of flashbev_sampling_vt_backward per frame, L2-cold frames."""
     from paper_2607_10071_b200 import binding as fb
     X, Y, Z = w.grid
     Hf, Wf = w.feat_hw
@@ -573,7 +573,7 @@ def main():
             print(json.dumps({"metric": "sampling_vt_backward_latency", "value": lat, "unit": "ms", "higher_is_better": False,
                               "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "dtype": "f32", "data": "synthetic",
                               "config": {"workload": wb.name, "C": wb.C, "grid": list(wb.grid), "feat_hw": list(wb.feat_hw),
-                                         "launch": "cuda graph replay, memset + scatter kernel per frame"},
+                                         "launch": "cuda graph replay, one backward call per frame"},
                               "gpu_launches": args.steps * max(4, -(-3 * L2_BYTES // (wb.output_bytes + wb.B * wb.N * wb.feat_hw[0] * wb.feat_hw[1] * wb.C * 4)))}))
         if world > 1:
             dist.destroy_process_group()

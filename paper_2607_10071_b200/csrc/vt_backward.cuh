@@ -22,7 +22,7 @@
 //
 // Why: the scatter hands two fp32 vector reductions per record to the crossbar -- 11.5 M sectors for a gradient of 0.17 M on
 // 200 x 200 x 8, C = 80 -- and is bound by the rate at which an SM can do that (92 us).  Here a texel leaves the SM once: 33 us;
-// 56 x 100 maps of tilted cameras, C = 128, Eq. 1: 144 -> 79 us.  What bounds it now: no unit (issue 34 %, tensor pipe 17 %); 16
+// 56 x 100 maps of tilted cameras, C = 128, Eq. 1: 144 -> 79 us.  What bounds it now: no unit (issue 30 %, L1 data pipe 22 %); 11 of at most 16
 // warps per SM that wait at the barriers of a round, for grad_out and for chains of fp64 operations, in 0.9 to 2 waves of CTAs of
 // unequal size.  128 registers: with 80 (24 warps per SM) the spills cost more than the warps bring
 // (calibrated 87 -> 116 us), but for up to 32 channels per warp (94 x 58 x 5, C = 32: 16.5 -> 13.4 us).
