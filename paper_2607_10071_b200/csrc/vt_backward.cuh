@@ -13,12 +13,15 @@
 //             the cell's column of a dense (row, cell) table in shared memory.  The mean modes count the cameras that see a bin by
 //             the signs of the validity conditions, and the factor is part of the weight.  For each tile of 16 rows a list says
 //             which cells have weights in it.
-//   products  gradient[row, channel] += weights[row, cell] x grad_out[cell, channel], 8 listed cells at a time on the tensor cores.
-//             Every fp32 number is the exact sum of two tf32 ones; three products (the fourth is below 2^-24 of the result) are
-//             summed from zero for these 8 cells and added to the accumulators in fp32.
+//   products  gradient[row, channel] += weights[row, cell] x grad_out[cell, channel], 16 listed cells at a time on the tensor cores.
+//             Every fp32 number is the exact sum of three bf16 ones.  The product of the leading pieces (16 bits: exact for one cell)
+//             and the sum of the five next ones are kept apart, and rounded to fp32 once, together; the three smallest are left out.
 //
-// Against fp64 the results are nearer than the scatter's (relative 2-norm 1.2e-7 to 1.5e-7 over 24 problems, the scatter
-// 1.9e-7 to 2.3e-7: long sums of reductions in any order).
+// A single product of a weight and a grad_out is off by at most 1.2e-7 of it, 2.6e-8 root mean square (an fp32 product: 6.0e-8 and
+// 2.5e-8).  Against fp64 the results are as near as the scatter's or nearer: relative 2-norm 5.8e-8 to 9.0e-8 over three problems, the
+// scatter 6.4e-8 to 2.2e-7 (long sums of reductions in any order), and 5.4e-8 to 6.3e-8 against 5.4e-8 to 6.5e-8 where two cells in a
+// hundred have a gradient.  Two tf32 pieces, a bit short of 24, and three products: 1.0e-7 to 1.4e-7 in all of them, single products
+// off by 4.8e-7, 7.8e-8 root mean square; 31.6 us on 200 x 200 x 8, C = 80, this 35.0.  Eight products (all but lo x lo) 39.6 us.
 //
 // Why: the scatter hands two fp32 vector reductions per record to the crossbar -- 11.5 M sectors for a gradient of 0.17 M on
 // 200 x 200 x 8, C = 80 -- and is bound by the rate at which an SM can do that (92 us).  Here a texel leaves the SM once: 33 us;
@@ -134,16 +137,25 @@ __device__ __forceinline__ void bwd_interval(const float (&a)[5], const float (&
     hi = empty ? -1 : min((int)floorf(fmaxf(h, -1.f) + guard), n - 1);
 }
 
-// v = hi + lo exactly, both with at most 11 significant bits
-__device__ __forceinline__ void split_tf32(float v, uint32_t &hi, uint32_t &lo)
+// a and b as sums of three bf16 numbers each, in pairs (a in the low half): 24 = 8 + 8 + 8 bits.  The differences are exact, and the
+// last piece has at most 7 bits left: nothing is lost.  With |v| in [1, 2) the pieces after the first are at most 2^-8 and 2^-17.
+// (Under 2^-109 the last bits fall below bf16's smallest number, 2^-133.  A number that rounds to infinity is one more
+// grad_out that is not finite: see the end of the kernel.)
+__device__ __forceinline__ void split_bf16(float a, float b, uint32_t &hi, uint32_t &mid, uint32_t &lo)
 {
-    hi = (__float_as_uint(v) + 0x1000u) & 0xffffe000u;
-    lo = __float_as_uint(v - __uint_as_float(hi));
+    const auto minus = [](uint32_t v) {
+        return make_float2(__uint_as_float((v << 16) ^ 0x80000000u), __uint_as_float((v & 0xffff0000u) ^ 0x80000000u));
+    };
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(b), "f"(a));
+    float2 r = __fadd2_rn(make_float2(a, b), minus(hi));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(mid) : "f"(r.y), "f"(r.x));
+    r = __fadd2_rn(r, minus(mid));
+    lo = __byte_perm(__float_as_uint(r.x), __float_as_uint(r.y), 0x7632u);
 }
 
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
+__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -391,31 +403,40 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                         const uint8_t *const slots = sm.slots + row_tile * 32 * warps;
                         const int n_slots = slots_n[row_tile];
 #pragma unroll 1
-                        for (int k = 8 * group; k < n_slots; k += 8 * q.groups) {
-                            // (cells past the last one: the last one, with weight 0)
-                            const int ka = k + (lane & 3), kb = ka + 4;
-                            const int sa = slots[min(ka, n_slots - 1)], sb = slots[min(kb, n_slots - 1)];
-                            const float *const pa = gout + (size_t)FB_IDX(sm.list[first + sa], p.X * p.Y, p.err) * (unsigned)p.C + ch0 + (lane >> 2);
-                            const float *const pb = gout + (size_t)FB_IDX(sm.list[first + sb], p.X * p.Y, p.err) * (unsigned)p.C + ch0 + (lane >> 2);
-                            float ga[NT], gb[NT];
+                        for (int k = 16 * group; k < n_slots; k += 16 * q.groups) {
+                            // (fragments: rows lane / 4 and + 8, cells 2 (lane % 4) and + 1, + 8, + 9.  Cells past the last one: the
+                            // last one, with weight 0)
+                            float g[4][NT], w[4][2];
 #pragma unroll
-                            for (int j = 0; j < NT; ++j) {
-                                const bool in = WHOLE || ch0 + 8 * j + (lane >> 2) < p.C;
-                                ga[j] = in ? __ldg(pa + 8 * j) : 0.f, gb[j] = in ? __ldg(pb + 8 * j) : 0.f;
+                            for (int c = 0; c < 4; ++c) {
+                                const int at = k + 2 * (lane & 3) + (c & 1) + (c >> 1) * 8, slot = slots[min(at, n_slots - 1)];
+                                const float *const src =
+                                    gout + (size_t)FB_IDX(sm.list[first + slot], p.X * p.Y, p.err) * (unsigned)p.C + ch0 + (lane >> 2);
+#pragma unroll
+                                for (int j = 0; j < NT; ++j)
+                                    g[c][j] = WHOLE || ch0 + 8 * j + (lane >> 2) < p.C ? __ldg(src + 8 * j) : 0.f;
+                                w[c][0] = at < n_slots ? wt[slot] : 0.f, w[c][1] = at < n_slots ? wt[8 * pitch + slot] : 0.f;
                             }
-                            uint32_t ah[4], al[4];
-                            split_tf32(ka < n_slots ? wt[sa] : 0.f, ah[0], al[0]), split_tf32(ka < n_slots ? wt[8 * pitch + sa] : 0.f, ah[1], al[1]);
-                            split_tf32(kb < n_slots ? wt[sb] : 0.f, ah[2], al[2]), split_tf32(kb < n_slots ? wt[8 * pitch + sb] : 0.f, ah[3], al[3]);
+                            uint32_t ah[4], am[4], al[4];
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) split_bf16(w[h & 2][h & 1], w[(h & 2) + 1][h & 1], ah[h], am[h], al[h]);
 #pragma unroll
                             for (int j = 0; j < NT; ++j) {
-                                uint32_t bh[2], bl[2];
-                                split_tf32(ga[j], bh[0], bl[0]), split_tf32(gb[j], bh[1], bl[1]);
-                                float t[4] = {0.f, 0.f, 0.f, 0.f};
-                                mma_tf32(t, al, bh[0], bh[1]);
-                                mma_tf32(t, ah, bl[0], bl[1]);
-                                mma_tf32(t, ah, bh[0], bh[1]);
-                                acc[i][j][0] = __fadd2_rn(acc[i][j][0], make_float2(t[0], t[1]));
-                                acc[i][j][1] = __fadd2_rn(acc[i][j][1], make_float2(t[2], t[3]));
+                                uint32_t bh[2], bm[2], bl[2];
+                                split_bf16(g[0][j], g[1][j], bh[0], bm[0], bl[0]);
+                                split_bf16(g[2][j], g[3][j], bh[1], bm[1], bl[1]);
+                                float t[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f};
+                                // (mid x lo, lo x mid and lo x lo are left out: at most 2^-24 of a product, 2^-27 root mean square)
+                                mma_bf16(t, ah, bh[0], bh[1]);
+                                mma_bf16(u, ah, bl[0], bl[1]);
+                                mma_bf16(u, al, bh[0], bh[1]);
+                                mma_bf16(u, am, bm[0], bm[1]);
+                                mma_bf16(u, ah, bm[0], bm[1]);
+                                mma_bf16(u, am, bh[0], bh[1]);
+                                const float2 s0 = __fadd2_rn(make_float2(t[0], t[1]), make_float2(u[0], u[1]));
+                                const float2 s1 = __fadd2_rn(make_float2(t[2], t[3]), make_float2(u[2], u[3]));
+                                acc[i][j][0] = __fadd2_rn(acc[i][j][0], s0);
+                                acc[i][j][1] = __fadd2_rn(acc[i][j][1], s1);
                             }
                         }
                     }

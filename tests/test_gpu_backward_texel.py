@@ -65,6 +65,35 @@ def test_many_cameras_see_every_cell(oracle):
         assert "texel" in check(oracle, w, inp.lidar2img, reduce)
 
 
+@pytest.mark.parametrize("C,feat,reduce", [(16, (20, 26), SUM), (32, (16, 22), SUM), (48, (18, 30), MEAN), (64, (32, 44), EQ1),
+                                           (80, (32, 44), SUM), (132, (30, 25), EQ1), (64, (47, 21), SUM), (128, (56, 50), EQ1)])
+def test_a_single_product_is_rounded_once(C, feat, reduce):
+    """Channels that one cell alone has a gradient in: two per cell, 1 in the one -- the result is the texel's weight, as it
+    stands in single precision -- and any number in the other, whose result is then one product.  It is rounded once (2^-24 of
+    it, half an ulp) and lacks the smallest products of its pieces (2^-24 at most); what the tensor cores cut off the others
+    is below 2^-27.  Root mean square: 2.53e-8 for the rounding (2^-24 / sqrt(3), over significands of 1 to 2), 0.6e-8 for the
+    rest, 2.6e-8 together; a thousand values are within a tenth of it."""
+    w = workload("single", C, feat, (40, 37, 5), reduce=reduce)
+    m = wl.make_inputs(w).lidar2img
+    rng = np.random.default_rng(C)
+    off = []
+    for _ in range(8):
+        G = np.zeros((1,) + tuple(w.grid[:2]) + (C,), np.float32)
+        g = (rng.uniform(1.0, 2.0, C // 2) * 2.0 ** rng.integers(-20, 20, C // 2) * rng.choice((-1, 1), C // 2)).astype(np.float32)
+        for c in range(C // 2):
+            x, y = rng.integers(w.grid[0]), rng.integers(w.grid[1])
+            G[0, x, y, 2 * c], G[0, x, y, 2 * c + 1] = 1.0, g[c]
+        got, name = run_backward(w, m, G, reduce)
+        assert "texel" in name
+        weight, result = got[..., 0::2].astype(np.float64), got[..., 1::2].astype(np.float64)
+        exact = weight * g.astype(np.float64)
+        assert np.array_equal(weight != 0.0, result != 0.0)
+        off.append(np.abs(result - exact)[weight != 0.0] / np.abs(exact[weight != 0.0]))
+    off = np.concatenate(off)
+    assert off.size > 1000
+    assert off.max() <= 2.0 ** -23 + 2.0 ** -27 and np.sqrt((off ** 2).mean()) <= 2.9e-8, (off.max(), np.sqrt((off ** 2).mean()))
+
+
 @pytest.mark.parametrize("shared", [False, True])
 def test_gradients_that_are_not_finite(shared):
     """Infinite and NaN output gradients reach the texels that their cell weighs and no others, as in the scatter."""
