@@ -28,6 +28,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <mutex>
 #include <type_traits>
 
@@ -1172,11 +1173,17 @@ flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, in
     const int rows = q.row_tiles * kBwdRows, channels = 8 * NT * q.ch_tiles;
     const int cblocks = (p->C + channels - 1) / channels, rblocks = (p->feat_h + rows - 1) / rows;
     const double columns = (double)p->B * p->N * p->feat_w * cblocks * rblocks;
-    // One CTA per column stores its sums, without a memset before and reductions after it.  Where that leaves SMs idle with long
-    // lists, two share a column.  One / two / three CTAs per column, us: 176 columns, 18 k cells, C = 96 23 / 20 / 23; 258, 28 k,
-    // C = 48 54 / 39 / 37; 276, 48 k, C = 32 29 / 26 / 32; but 252, 12 k, C = 96 17 / 29 / 37, 290, 12 k, C = 48 28 / 27 / 31, and
-    // 528, 40 k, C = 80 33 / 37 / 39.
-    q.slices = columns <= 2.0 * sm_count() && (double)p->X * p->Y > 100.0 * p->N * p->feat_w ? 2 : 1;
+    // One CTA per column stores its sums, without a memset before and reductions after it.  Where that leaves the SMs empty, as many
+    // share a column as the SMs hold at once (16 warps of 128 registers each), up to eight, while each still has 20 cells: a camera
+    // sees about a fifth of a grid around it.  With long lists two share it even if half of them wait.  Scatter / one / two / four /
+    // eight CTAs per column, us: 28 columns, 50 k cells, C = 128 35 / 86 / 50 / 30 / 21; 56 of C = 48 over 63 k 33 / 51 / 31 / 23 / 17;
+    // 102 of C = 128 (two in SMs that hold two) over 78 k 142 / 135 / 77 / 67 / 63; but 138 of C = 128 over 98 k 77 / 34 / 25 / 32 / 47,
+    // 290 of C = 96 over 8 k 33 / 16 / 17 / 25 / 41.  Over 180 calls of 20 to 640 columns the best of 1 to 16 CTAs is 5 % faster
+    // (geometric mean; two at most: 21 %), the scatter 7 % at most (42 %).
+    const int resident = kBwdSmWarps / (q.row_warps * q.ch_tiles * q.groups) * sm_count();
+    const double cells = (double)p->X * p->Y / p->feat_w;
+    const bool two = columns <= 2.0 * sm_count() && cells > 100.0 * p->N;
+    q.slices = (int)std::max(two ? 2.0 : 1.0, std::min({8.0, std::floor(resident / columns), std::floor(cells / std::max(p->N, 5) / 20.0)}));
     q.exclusive = q.slices == 1;
     smem = bwd_smem_layout(nullptr, nullptr, p->N, q.row_tiles, q.row_warps, q.ch_tiles, q.groups, NT, RT, p->reduce);
     const double blocks = (double)p->B * p->N * p->feat_w * q.slices;

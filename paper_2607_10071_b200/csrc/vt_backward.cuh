@@ -33,7 +33,8 @@
 
 constexpr int kBwdRows = 16;       // texel rows of a warp's tile
 constexpr int kBwdMaxTiles = 4;    // ... times this many per CTA
-constexpr int kBwdMaxWarps = 8;
+constexpr int kBwdMaxWarps = 8;    // of a CTA
+constexpr int kBwdSmWarps = 16;    // that an SM holds (24 in the instances of 80 registers)
 constexpr int kBwdList = 1024;     // cells that wait for their weights
 constexpr int kBwdDeal = 8;        // cells along y that go to the same slice
 
