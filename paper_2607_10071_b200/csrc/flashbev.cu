@@ -967,7 +967,7 @@ cudaError_t launch_tiled_warps(int warps, const KParams &k, dim3 grid, size_t sm
                 if (V % 2 == 0 && k.wide) return launch_tiled_inst<V, BF16, 4, false, (V % 2 == 0), true>(k, grid, smem, stream);
                 return launch_tiled_inst<V, BF16, 4, false, false, true>(k, grid, smem, stream);
             }
-            if (k.level && (V > 1 || BF16)) {  // (instances for 4 warps per CTA only)
+            if (k.level && (V > 1 || BF16)) {  // (of 4 warps per CTA; the others take levels too)
                 if (V % 2 == 0 && k.wide) return launch_tiled_inst<V, BF16, 4, false, (V % 2 == 0), false, true>(k, grid, smem, stream);
                 return launch_tiled_inst<V, BF16, 4, false, false, false, true>(k, grid, smem, stream);
             }
@@ -1126,9 +1126,7 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
     int V, warps;
     dim3 grid;
     size_t smem;
-    flashbev_vt_params q = *p;
-    if (pyramid) q.tune[3] = (q.tune[3] & ~0xf) | 4;  // the instances for pyramid levels are built for 4 warps per CTA
-    const flashbev_status st = configure_tiled(&q, k, V, warps, grid, smem, accumulate, false, scalar_out == 1);
+    const flashbev_status st = configure_tiled(p, k, V, warps, grid, smem, accumulate, false, scalar_out == 1);
     if (st != FLASHBEV_OK) return st;
     k.out_nchw = scalar_out != 0;
     {

@@ -106,6 +106,31 @@ def test_levels_accumulate_in_order_and_ignore_what_out_held():
     assert torch.equal(out, first + added)
 
 
+@pytest.mark.parametrize("dtype,C", [("f32", 32), ("f32", 80), ("f32", 96), ("f32", 224), ("bf16", 64), ("bf16", 128), ("bf16", 320)])
+def test_warps_per_cta_are_honoured(dtype, C):
+    """The hint for the warps of a CTA reaches the kernels of the levels: sums are the same bit for bit, and eight warps whose
+    record slots do not fit an SM's shared memory are refused as in the call for one map."""
+    import torch
+    w = wl.Workload(f"mrw{C}", 5300 + C, 1, 6, C, dtype, (20, 36), (160, 288), (41, 37, 8), (-25.0, 25.0, -25.0, 25.0, -4.0, 3.0), 0)
+    feats, bits, mats = wl.make_pyramid_inputs(w, 3)
+    f, m = _upload(w, feats, bits, mats)
+    args = (w.img_hw, w.bev_range, w.grid, EQ1)
+
+    def pyramid(hint, levels=f):
+        return fb.sampling_vt_multires(levels, m, *args, kernel=fb.KERNEL_TILED, tune=(0, 0, 0, hint))
+
+    want = pyramid(4)
+    for warps in (1, 2, 8):
+        assert torch.equal(pyramid(warps), want), warps
+    slots = 160 << 20  # 2560 records of 12 bytes per warp
+    assert torch.isfinite(pyramid(4 | slots)).all()
+    for call in (lambda: fb.sampling_vt(f[0], m, *args, kernel=fb.KERNEL_TILED, tune=(0, 0, 0, 8 | slots)), lambda: pyramid(8 | slots),
+                 lambda: pyramid(8 | slots, f[:1])):
+        with pytest.raises(fb.FlashBevError) as e:
+            call()
+        assert e.value.status == fb.UNSUPPORTED
+
+
 def test_rejections():
     import torch
     w = wl.get("tiny")
