@@ -1194,8 +1194,12 @@ template <int NT, int RT = 1>
 cudaError_t launch_backward(const BwdParams &q, dim3 grid, size_t smem, cudaStream_t stream)
 {
     const bool sum = q.k.reduce == FLASHBEV_REDUCE_SUM, full = q.k.C == (int)grid.y * q.ch_tiles * 8 * NT;
-    const auto kernel = sum ? (full ? vt_texel_backward_kernel<NT, RT, true, true> : vt_texel_backward_kernel<NT, RT, true, false>)
-                            : (full ? vt_texel_backward_kernel<NT, RT, false, true> : vt_texel_backward_kernel<NT, RT, false, false>);
+    auto kernel = full ? vt_texel_backward_kernel<NT, RT, true, true> : vt_texel_backward_kernel<NT, RT, true, false>;
+    if constexpr (NT > 4 || (NT == 4 && RT == 2)) {
+        if (!sum) kernel = full ? vt_texel_backward_kernel<NT, RT, false, true> : vt_texel_backward_kernel<NT, RT, false, false>;
+    } else if (!sum) {
+        return cudaErrorNotSupported;  // (the mean modes come with more than 40 channels only: backward_by_texel)
+    }
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;

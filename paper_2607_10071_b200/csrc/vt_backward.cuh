@@ -43,7 +43,6 @@ struct BwdParams {
     int row_tiles;                    // tiles of 16 rows per CTA
     int row_warps, ch_tiles, groups;  // warps of a CTA: groups of row_warps x ch_tiles; a warp has every row_warps-th row tile
     int slices;                       // CTAs that share a texel column, each with its share of the cells
-    int first_map;                    // the first b * N + n of the launch
     int exclusive;                    // one CTA per column: results are stored, not added
 };
 
@@ -183,9 +182,8 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
 
     // ---- which texel column (rows from blockIdx.z on, channels from blockIdx.y on)
     const unsigned column = blockIdx.x / (unsigned)q.slices, slice = blockIdx.x - column * (unsigned)q.slices;
-    const unsigned cam = column / (unsigned)p.Wf;
-    const unsigned map = cam + (unsigned)q.first_map;  // b * N + n
-    const int xt = (int)(column - cam * (unsigned)p.Wf);
+    const unsigned map = column / (unsigned)p.Wf;  // b * N + n
+    const int xt = (int)(column - map * (unsigned)p.Wf);
     const int rows = q.row_tiles * kBwdRows, ya = blockIdx.z * rows, rv = min(rows, p.Hf - ya), pitch = 32 * warps + 4;
     const int b = (int)(map / (unsigned)p.N), n = (int)(map - (unsigned)b * p.N);
     const size_t rowf = (size_t)p.Wf * p.C;
