@@ -1160,10 +1160,12 @@ flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, in
     q.k = base_params(p);
     q.row_tiles = std::min(kBwdMaxTiles, (p->feat_h + kBwdRows - 1) / kBwdRows);
     // Three or four row tiles: the middle ones, about the horizon, have most of the cells, so a warp takes two of them, a long and a
-    // short one, and half the channels -- unless its 32 channels pad the call's to more than tiles of 80 do: then the products of the
-    // padding cost more.  Two row tiles per warp, as time over that of one, six maps of 33 to 64 rows, level and tilted, SUM and Eq. 1:
-    // C = 64 0.93 (0.81 to 1.24), 96 0.99 (0.90 to 1.06), 112 0.92 (0.81 to 1.02), 128 0.89 (0.73 to 1.01); 56 x 100, C = 128, tilted,
-    // Eq. 1 82 us against 90.  But C = 44 1.10 (0.98 to 1.56), 48 1.12 (0.96 to 1.56), 80 1.04 (0.85 to 1.35; 38 x 56 48 us against 38).
+    // short one, and half the channels -- unless its 32 channels pad the call's by a quarter more than tiles of 80 do (36 to 48
+    // channels): the products of the padding cost more then.  Two row tiles per warp, as time over that of one (geometric mean and
+    // range of 18 to 24 calls, six maps of 33 to 64 rows, level and tilted): C = 64 0.93 (0.81-1.24), 80 1.04 (0.85-1.35), 96 0.99
+    // (0.90-1.06), 112 0.92 (0.81-1.02), 128 0.89 (0.73-1.01; 56 x 100, tilted, Eq. 1 82 us against 90), but 44 1.10 (0.98-1.56), 48
+    // 1.12 (0.96-1.56; 38 x 56, level, SUM 41 us against 28).  80 stays with two for its worst cases (60 x 50, 300 x 200 x 16, Eq. 1
+    // 156 us against 183).
     const auto padded = [&](int most, int &tiles, int &nt) {
         tiles = (p->C + most - 1) / most;
         nt = ((p->C + tiles - 1) / tiles + 15) / 16 * 2;  // (instances for every other NT)
@@ -1171,7 +1173,7 @@ flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, in
     };
     int ch_tiles, narrow_tiles, narrow;
     const int wide = padded(80, ch_tiles, NT);
-    RT = q.row_tiles > 2 && p->C <= 128 && padded(32, narrow_tiles, narrow) <= wide ? 2 : 1;
+    RT = q.row_tiles > 2 && p->C <= 128 && 4 * padded(32, narrow_tiles, narrow) <= 5 * wide ? 2 : 1;
     if (RT == 2) ch_tiles = narrow_tiles, NT = narrow;
     q.row_warps = (q.row_tiles + RT - 1) / RT;
     q.ch_tiles = std::min(ch_tiles, kBwdMaxWarps / q.row_warps);

@@ -37,7 +37,7 @@ def test_channel_tiles(oracle, C):
 @pytest.mark.parametrize("C", [4, 32, 36, 48, 64, 80, 100, 128, 132])
 @pytest.mark.parametrize("rows", [33, 48, 49, 64])
 def test_two_row_tiles_per_warp(oracle, C, rows):
-    """Three and four row tiles: up to 128 channels a warp has two of them, unless that pads the channels further (36, 48, 80)."""
+    """Three and four row tiles: up to 128 channels a warp has two of them, unless that pads the channels much further (36, 48)."""
     w = workload("two_tiles", C, (rows, 14), (23, 27, 12), general=C % 8 == 0, N=4)
     assert "texel" in check(oracle, w, wl.make_inputs(w).lidar2img, SUM, seed=rows)
 
