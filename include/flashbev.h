@@ -214,10 +214,10 @@ flashbev_status flashbev_sampling_vt_host_static(const flashbev_vt_params *p, vo
  * 1/max(1, valid samples of the cell) (MEAN_OVER_VALID), 1/max(1, cameras seeing that height bin)
  * (CAMERA_MEAN_Z_SUM).  Geometry fields have the meaning they have in flashbev_vt_params.
  *
- * Enqueues one kernel on `stream` that takes the sums texel by texel, or (few channels over many cells, more than 64 height
- * bins, launch hints in `tune`) a memset of `grad_features` to zero and one that scatters with fp32 vector atomics.  The
- * summation order -- and the last bits of the result -- can differ from run to run.  Allocates nothing.  C must be a multiple of
- * 4 and both gradient pointers 16-byte aligned, else FLASHBEV_UNSUPPORTED / FLASHBEV_MISALIGNED.
+ * Enqueues one kernel on `stream` that takes the sums texel by texel (after a memset of `grad_features` to zero where there are
+ * so few texel columns that several blocks share one), or (few channels over many cells, more than 64 height bins, launch hints
+ * in `tune`) a memset and a kernel that scatters with fp32 vector atomics.  The summation order -- and the last bits of the
+ * result -- can differ from run to run.  Allocates nothing.  C must be a multiple of 4 and both gradient pointers 16-byte aligned, else FLASHBEV_UNSUPPORTED / FLASHBEV_MISALIGNED.
  */
 typedef struct flashbev_vt_backward_params {
     size_t struct_size;        /* sizeof(flashbev_vt_backward_params) of the caller's header */

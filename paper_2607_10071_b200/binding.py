@@ -283,7 +283,7 @@ def make_backward_params(grad_out_ptr, lidar2img_ptr, B, N, C, feat_hw, img_hw, 
 
 def flashbev_sampling_vt_backward(params: VtBackwardParams, stream: int | None = None, check: bool = True,
                                   library=None) -> int:
-    """Enqueue the gradient w.r.t. the features (memset + one scatter kernel) on ``stream``."""
+    """Enqueue the gradient w.r.t. the features (one kernel, after a memset where blocks share texels) on ``stream``."""
     st = (library or lib()).flashbev_sampling_vt_backward(ctypes.byref(params), ctypes.c_void_p(stream or 0))
     if check and st != OK:
         raise FlashBevError(st, "flashbev_sampling_vt_backward")

@@ -1191,7 +1191,8 @@ flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, in
     const int resident = kBwdSmWarps / (q.row_warps * q.ch_tiles * q.groups) * sm_count();
     const double cells = (double)p->X * p->Y / p->feat_w;
     const bool two = columns <= 2.0 * sm_count() && cells > 100.0 * p->N;
-    q.slices = (int)std::max(two ? 2.0 : 1.0, std::min({8.0, std::floor(resident / columns), std::floor(cells / std::max(p->N, 5) / 20.0)}));
+    const double most = std::min({8.0, std::floor(resident / columns), std::floor(cells / std::max(p->N, 5) / 20.0)});
+    q.slices = (int)std::max(two ? 2.0 : 1.0, most);
     q.exclusive = q.slices == 1;
     smem = bwd_smem_layout(nullptr, nullptr, p->N, q.row_tiles, q.row_warps, q.ch_tiles, q.groups, NT, RT, p->reduce);
     const double blocks = (double)p->B * p->N * p->feat_w * q.slices;
@@ -1220,11 +1221,15 @@ cudaError_t launch_backward(const BwdParams &q, dim3 grid, size_t smem, cudaStre
 // Which of the two backward kernels takes a call: the texel-side one, but not
 // - with hints, which are launch geometry of the scatter;
 // - with more than 64 height bins, each of which it projects (the scatter solves for intervals);
-// - with few channels, unless in SUM mode on few cells: it makes its geometry, and the mean modes their counts, for every texel
-//   column that a cell reaches, whatever the channels.  Scatter / texel side, us, C = 32, tilted cameras: Eq. 1 on 37 k cells 56 / 95,
-//   63 k 103 / 147; mean on 6 k 18 / 25, 10 k 23 / 25; SUM on 19 k 36 / 42, 28 k 64 / 59, but 6 k 16 / 12, 14 k 33 / 21, 9 k 23 / 17.
-// From 48 channels on it wins: 44 of 46 measured calls by up to 2.8x (geometric mean 1.55; 200 x 200 x 8, C = 80 92 / 33, C = 128 on
-// tilted cameras 143 / 87), the others 45 / 47 and 30 / 29.
+// - with up to 40 channels, unless in SUM mode on few cells: it makes its geometry, and the mean modes their counts, for every texel
+//   column that a cell reaches, whatever the channels.  Scatter / texel side, us in a graph, six tilted cameras, 32 x 88 maps, 8 bins,
+//   6 k, 20 k and 62 k cells: C = 32 SUM 14 / 12, 27 / 28, 57 / 72, mean 14 / 14, 27 / 33, 57 / 89, Eq. 1 14 / 14, 28 / 32, 58 / 82;
+//   C = 16 SUM 13 / 10, 21 / 21, 43 / 53; C = 8 SUM 12 / 10, 18 / 22, 34 / 56.  The line in cells, 50 per texel column, loses a
+//   quarter at the most against the better one of the two (16 x 44 maps, C = 32, SUM: 10 k cells 15 / 18, 20 k 22 / 18).  At C = 40,
+//   where the scatter's lanes divide badly, the texel side would win in all three modes (19 / 10, 37 / 22, 83 / 58 in SUM).
+// Above 40 channels it wins: 54 of 60 drawn calls of 48 to 256 channels, by up to 3.2x (geometric mean 1.50; 200 x 200 x 8, C = 80
+// 87 / 34, C = 128 on tilted cameras, Eq. 1 137 / 88); the others take up to 1.13 times as long, one of them 1.27 times (C = 64,
+// 55 x 144 maps, 75 x 53 x 4 cells: 15 / 19).
 bool backward_by_texel(const flashbev_vt_params *p)
 {
     for (int t : p->tune)
@@ -1286,7 +1291,8 @@ flashbev_status launch_nchw_tiled(const flashbev_vt_params *p, cudaStream_t stre
     const dim3 grid((unsigned)((HW + 64 * E - 1) / (64 * E)), (unsigned)((q.C + 4 * E - 1) / (4 * E)), (unsigned)(p->B * p->N));
     auto copy = [&](auto kernel, auto *elem) {
         using T = typename std::remove_pointer<decltype(elem)>::type;
-        launch_dependent(kernel, grid, dim3(256), 0, stream, static_cast<const T *>(p->features), static_cast<T *>(p->workspace), p->C, q.C, HW);
+        launch_dependent(kernel, grid, dim3(256), 0, stream, static_cast<const T *>(p->features), static_cast<T *>(p->workspace), p->C,
+                         q.C, HW);
     };
     if (E == 8 && aligned) copy(nchw_to_nhwc_kernel<uint16_t, true>, (uint16_t *)nullptr);
     else if (E == 8) copy(nchw_to_nhwc_kernel<uint16_t, false>, (uint16_t *)nullptr);

@@ -5,31 +5,35 @@
 // in registers (a warp: 16 rows by 8 NT channels, as the accumulators of m16n8 fragments) while the CTA goes through the BEV
 // cells that reach the column, in rounds of 32 cells per warp:
 //
-//   survey    The cells in question.  Depth and the limits of the column and of its rows are linear functions of the position that
-//             must be positive wherever the depth is.  A lane takes a grid row (one x) and solves for the interval of y in which
-//             the largest value of each over the heights is not negative; the warp numbers the intervals' cells through and
-//             appends them to the CTA's list, 32 at a time.
-//   weights   A lane takes a cell: it projects the height bins that can reach the column in fp64 and adds their bilinear weights to
-//             the cell's column of a dense (row, cell) table in shared memory.  The mean modes count the cameras that see a bin by
-//             the signs of the validity conditions, and the factor is part of the weight.  For each tile of 16 rows a list says
-//             which cells have weights in it.
-//   products  gradient[row, channel] += weights[row, cell] x grad_out[cell, channel], 16 listed cells at a time on the tensor cores.
-//             Every fp32 number is the exact sum of three bf16 ones.  The product of the leading pieces (16 bits: exact for one cell)
-//             and the sum of the five next ones are kept apart, and rounded to fp32 once, together; the three smallest are left out.
+//   survey    The cells in question.  Depth and the limits of the column and of its rows are linear functions of the position
+//             that must be positive wherever the depth is.  A lane takes a grid row (one x) and solves for the interval of y in
+//             which the largest value of each over the heights is not negative; the warp numbers the intervals' cells through
+//             and appends them to the CTA's list, 32 at a time.
+//   weights   A lane takes a cell: it projects the height bins that can reach the column in fp64 and adds their bilinear weights
+//             to the cell's column of a dense (row, cell) table in shared memory.  The mean modes count the cameras that see a
+//             bin by the signs of the validity conditions, and the factor is part of the weight.  For each tile of 16 rows a
+//             list says which cells have weights in it.
+//   products  gradient[row, channel] += weights[row, cell] x grad_out[cell, channel], 16 listed cells at a time on the tensor
+//             cores.  Every fp32 number is the exact sum of three bf16 ones.  The product of the leading pieces (16 bits: exact
+//             for one cell) and the sum of the five next ones are kept apart, and rounded to fp32 once, together; the three
+//             smallest are left out.
 //
 // A single product of a weight and a grad_out is off by at most 1.2e-7 of it, 2.6e-8 root mean square (an fp32 product: 6.0e-8 and
-// 2.5e-8).  Against fp64 the results are as near as the scatter's or nearer: relative 2-norm 5.8e-8 to 9.0e-8 over three problems, the
-// scatter 6.4e-8 to 2.2e-7 (long sums of reductions in any order), and 5.4e-8 to 6.3e-8 against 5.4e-8 to 6.5e-8 where two cells in a
-// hundred have a gradient.  Two tf32 pieces, a bit short of 24, and three products: 1.0e-7 to 1.4e-7 in all of them, single products
-// off by 4.8e-7, 7.8e-8 root mean square; 31.6 us on 200 x 200 x 8, C = 80, this 35.0.  Eight products (all but lo x lo) 39.6 us.
+// 2.5e-8).  Against fp64 the results are as near as the scatter's or nearer: relative 2-norm 5.8e-8 to 9.0e-8 over three problems,
+// the scatter 6.4e-8 to 2.2e-7 (long sums of reductions in any order), and 5.4e-8 to 6.3e-8 against 5.4e-8 to 6.5e-8 where two cells
+// in a hundred have a gradient.  Two tf32 pieces, a bit short of 24, and three products: 1.0e-7 to 1.4e-7 in all of them, single
+// products off by 4.8e-7, 7.8e-8 root mean square; 31.5 us on 200 x 200 x 8, C = 80, this 35.0.  Eight products (all but lo x lo)
+// 39.6 us.
 //
 // Why: the scatter hands two fp32 vector reductions per record to the crossbar -- 11.5 M sectors for a gradient of 0.17 M on
-// 200 x 200 x 8, C = 80 -- and is bound by the rate at which an SM can do that (92 us).  Here a texel leaves the SM once: 33 us;
-// 56 x 100 maps of tilted cameras, C = 128, Eq. 1: 144 -> 79 us.  What bounds it now: no unit (issue 30 %, L1 data pipe 22 %); 11 of at most 16
-// warps per SM that wait at the barriers of a round, for grad_out and for chains of fp64 operations, in 0.9 to 2 waves of CTAs of
-// unequal size.  128 registers: with 80 (24 warps per SM) the spills cost more than the warps bring
-// (calibrated 87 -> 116 us), but for up to 32 channels per warp (94 x 58 x 5, C = 32: 16.5 -> 13.4 us).
-// Row tiles of 32 rows without lists 37 and 116 us; fp32 FMAs instead of fragments 48 and 88 us (row quads) or slower.
+// 200 x 200 x 8, C = 80 -- and is bound by the rate at which an SM can do that.  Here a texel leaves the SM once: 92 -> 35 us a pass
+// (in a graph, into one result buffer, 87 -> 34); 56 x 100 maps of tilted cameras, C = 128, Eq. 1: 141 -> 88 us (137 -> 88).
+// What bounds it now: no unit (on these two, of the SMs' active cycles: issue 38 and 45 %, tensor pipe 19 %; L1 data pipe 25 and 35 %
+// of the launch); 12 and 15 of at most 16 warps per SM that wait at the barriers of a round, for grad_out and for chains of fp64
+// operations, in 0.9 and 2 waves of CTAs of unequal size: an SM is active for 72 and 77 % of the launch.
+// Forms that lost (measured with the tf32 products): 80 registers (24 warps per SM), whose spills cost more than the warps bring
+// (calibrated 87 -> 116 us), but for up to 32 channels per warp (94 x 58 x 5, C = 32: 16.5 -> 13.4 us); row tiles of 32 rows without
+// lists 37 and 116 us; fp32 FMAs instead of fragments 48 and 88 us (row quads) or slower.
 
 constexpr int kBwdRows = 16;       // texel rows of a warp's tile
 constexpr int kBwdMaxTiles = 4;    // ... times this many per CTA
@@ -64,8 +68,8 @@ struct BwdSmem {
     uint8_t *slots;        // [row_tiles][32 warps]: the round's cells that have weights in the row tile
 };
 
-__host__ __device__ inline size_t bwd_smem_layout(unsigned char *base, BwdSmem *t, int N, int row_tiles, int row_warps, int ch_tiles, int groups,
-                                                  int NT, int RT, int reduce)
+__host__ __device__ inline size_t bwd_smem_layout(unsigned char *base, BwdSmem *t, int N, int row_tiles, int row_warps, int ch_tiles,
+                                                  int groups, int NT, int RT, int reduce)
 {
     size_t o = 0;
     auto take = [&](size_t bytes) {
@@ -85,7 +89,8 @@ __host__ __device__ inline size_t bwd_smem_layout(unsigned char *base, BwdSmem *
     unsigned char *p6 = take((size_t)row_tiles * 32 * warps);
     if (t) {
         t->weights = reinterpret_cast<float *>(p0), t->mats = reinterpret_cast<double *>(p1);
-        t->exact = reinterpret_cast<double(*)[4]>(p2), t->tile = reinterpret_cast<BwdCond *>(p3), t->sees = reinterpret_cast<BwdCond *>(p4);
+        t->exact = reinterpret_cast<double(*)[4]>(p2);
+        t->tile = reinterpret_cast<BwdCond *>(p3), t->sees = reinterpret_cast<BwdCond *>(p4);
         t->list = reinterpret_cast<uint32_t *>(p5), t->slots = p6;
     }
     return o;
@@ -100,8 +105,8 @@ __device__ __forceinline__ BwdCond bwd_condition(const KParams &p, const double 
     const float lim = t == 1 ? fmaxf(x0, -0.5f) + 0.5f - eps : t == 2 ? fminf(x1, (float)p.Wf - 0.5f) + 0.5f + eps
                     : t == 3 ? fmaxf(y0, -0.5f) + 0.5f - eps : fminf(y1, (float)p.Hf - 0.5f) + 0.5f + eps;
     const float zl = (float)(p.z_min + 0.5 * p.dz), zs = (float)p.dz * (float)(p.Z - 1);
-    const float most[4] = {(float)fmax(fabs(p.x_min), fabs(p.x_min + p.dx * p.X)), (float)fmax(fabs(p.y_min), fabs(p.y_min + p.dy * p.Y)),
-                           fmaxf(fabsf(zl), fabsf(zl + zs)), 1.f};
+    const float most[4] = {(float)fmax(fabs(p.x_min), fabs(p.x_min + p.dx * p.X)),
+                           (float)fmax(fabs(p.y_min), fabs(p.y_min + p.dy * p.Y)), fmaxf(fabsf(zl), fabsf(zl + zs)), 1.f};
     float u[4], err = 0.f;  // the coefficients of (x, y, z, 1)
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -160,9 +165,9 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// NT: channels per warp / 8.  RT: row tiles per warp.  SUM: the reduce mode without counts of other cameras.  WHOLE: the channels fill the warps' tiles (a quarter
-// of the products' instructions would be checks).  (Every stage is in the kernel once and small:
-// a CTA runs most of it once, through an instruction cache that it shares with others at other stages.)
+// NT: channels per warp / 8.  RT: row tiles per warp.  SUM: the reduce mode without counts of other cameras.  WHOLE: the channels
+// fill the warps' tiles (a quarter of the products' instructions would be checks).  (Every stage is in the kernel once and small: a
+// CTA runs most of it once, through an instruction cache that it shares with others at other stages.)
 template <int NT, int RT, bool SUM, bool WHOLE>
 __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_texel_backward_kernel(const BwdParams q)
 {
@@ -228,16 +233,18 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
     const int ch0 = (blockIdx.y * q.ch_tiles + warp % q.ch_tiles) * (NT * 8);
     float2 acc[RT][NT][2];  // fragment layout: rows lane / 4 and + 8, channels 2 (lane % 4) and + 1
     const float *const gout = p.gout + (size_t)b * p.X * p.Y * p.C;
-    const float x_first = (float)(p.x_min + 0.5 * p.dx), y_first = (float)(p.y_min + 0.5 * p.dy), dxf = (float)p.dx, dyf = (float)p.dy;
+    const float x_first = (float)(p.x_min + 0.5 * p.dx), y_first = (float)(p.y_min + 0.5 * p.dy);
+    const float dxf = (float)p.dx, dyf = (float)p.dy;
 #pragma unroll
     for (int i = 0; i < RT; ++i)
 #pragma unroll
         for (int j = 0; j < NT; ++j) acc[i][j][0] = acc[i][j][1] = make_float2(0.f, 0.f);
     // (a second pass, if a grad_out that is not finite was met: see the end)
     for (bool again = false;; again = true) {
-        int row0 = 32 * (warp - warps);           // a chunk is 32 grid rows, a row per lane
-        int y_lo = 0, y_n = 0, y_sum = 0;         // the lane's row: first cell, cells, cells up to the end of it
-        unsigned chunk_n = 0, next = 0, sl = (slice + (unsigned)warp) % (unsigned)q.slices;  // cells of the chunk; this slice's next one
+        int row0 = 32 * (warp - warps);    // a chunk is 32 grid rows, a row per lane
+        int y_lo = 0, y_n = 0, y_sum = 0;  // the lane's row: first cell, cells, cells up to the end of it
+        unsigned chunk_n = 0, next = 0;    // cells of the chunk; this slice's next one
+        unsigned sl = (slice + (unsigned)warp) % (unsigned)q.slices;
 
         for (bool done = false;;) {
             // ---- survey: cells that can reach the column, until the list is full
@@ -270,7 +277,8 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                     sl = sl + 1u >= (unsigned)q.slices ? 0u : sl + 1u;
                     continue;
                 }
-                if (*(volatile int *)&list_n > kBwdList - 32 * warps) break;  // (every warp may add 32 cells before it sees another's)
+                // (every warp may add 32 cells before it sees another's)
+                if (*(volatile int *)&list_n > kBwdList - 32 * warps) break;
                 const bool keep = j < chunk_n;
                 int r = 0;  // the first row whose cells end behind j
 #pragma unroll
@@ -283,7 +291,8 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                 int at = 0;
                 if (lane == 0) at = atomicAdd(&list_n, __popc(bal));
                 at = __shfl_sync(FULL, at, 0);
-                if (keep) sm.list[FB_IDX(at + __popc(bal & lt_mask), kBwdList, p.err)] = FB_IDX((row0 + r) * p.Y + iy, p.X * p.Y, p.err);
+                at += __popc(bal & lt_mask);
+                if (keep) sm.list[FB_IDX(at, kBwdList, p.err)] = FB_IDX((row0 + r) * p.Y + iy, p.X * p.Y, p.err);
                 next += 32;
             }
             const bool all_done = __syncthreads_and(done);
@@ -293,7 +302,10 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                 if (first + 32 * warp < waiting) {
                     // ---- weights of 32 cells, a cell per lane
                     float *const own = sm.weights + 32 * warp + lane;
-                    for (int i = lane; i < rows * 8; i += 32) *reinterpret_cast<float4 *>(sm.weights + 32 * warp + (i >> 3) * pitch + (i & 7) * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int i = lane; i < rows * 8; i += 32) {
+                        float *const at = sm.weights + 32 * warp + (i >> 3) * pitch + (i & 7) * 4;
+                        *reinterpret_cast<float4 *>(at) = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
                     __syncwarp();
                     unsigned touched = 0u;  // bit t: the cell has weights in row tile t
                     if (first + 32 * warp + lane < waiting) {
@@ -338,8 +350,10 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                             }
                             if (!eq1) {
                                 int count = 0;
-                                for (unsigned long long s = seen; s; s &= s - 1ull)
-                                    for (int k = 0; k < p.Z; k += 4) count += __popc(bins(__ffsll((long long)s) - 1, k, min(4, p.Z - k)));
+                                for (unsigned long long s = seen; s; s &= s - 1ull) {
+                                    const int m = __ffsll((long long)s) - 1;
+                                    for (int k = 0; k < p.Z; k += 4) count += __popc(bins(m, k, min(4, p.Z - k)));
+                                }
                                 scale = 1.f / (float)max(count, 1);
                             }
                         }
@@ -347,7 +361,8 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                         const double a1 = fma(M[5], xy.y, fma(M[4], xy.x, M[7]));
                         const double a2 = fma(M[9], xy.y, fma(M[8], xy.x, M[11]));
                         const double wlim = (double)p.Wf - 0.5, hlim = (double)p.Hf - 0.5;
-                        constexpr int K = NT * RT <= 4 ? 2 : 4;  // bins projected together: a projection is a chain of a dozen fp64 operations
+                        // bins projected together: a projection is a chain of a dozen fp64 operations
+                        constexpr int K = NT * RT <= 4 ? 2 : 4;
                         for (int k0 = klo; k0 <= khi; k0 += K) {
                             int rr[K];
                             float wx[K], ty[K];
@@ -356,7 +371,8 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                                 const double zw = fma((double)(k0 + j), p.dz, zl);
                                 const double d = fma(M[10], zw, a2), r = fast_rcp(d);  // (d <= 0 and NaN fail below)
                                 const double fx = fma(fma(M[2], zw, a0), r, -0.5), fy = fma(fma(M[6], zw, a1), r, -0.5);
-                                bool ok = (k0 + j <= khi) & (d > kDepthMin) & (fx > -0.5) & (fx < wlim) & (fy > -0.5) & (fy < hlim);
+                                bool ok = (k0 + j <= khi) & (d > kDepthMin);
+                                ok &= (fx > -0.5) & (fx < wlim) & (fy > -0.5) & (fy < hlim);
                                 double flx, fly;
                                 const int c = floor_int(fx, flx) - xt, row = floor_int(fy, fly) - ya;
                                 const float tx = (float)(fx - flx);
@@ -377,8 +393,14 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                                 if (r < -1) continue;
                                 const float sc = eq1 ? 1.f / (float)(1u + ((den >> (8 * j)) & 0xffu)) : scale;
                                 const float w = wx[j] * sc;
-                                if (r >= 0) own[FB_IDX(r, rows, p.err) * pitch] += w * (1.f - ty[j]), touched |= 1u << (r / kBwdRows);
-                                if (r + 1 < rv) own[FB_IDX(r + 1, rows, p.err) * pitch] += w * ty[j], touched |= 1u << ((r + 1) / kBwdRows);
+                                if (r >= 0) {
+                                    own[FB_IDX(r, rows, p.err) * pitch] += w * (1.f - ty[j]);
+                                    touched |= 1u << (r / kBwdRows);
+                                }
+                                if (r + 1 < rv) {
+                                    own[FB_IDX(r + 1, rows, p.err) * pitch] += w * ty[j];
+                                    touched |= 1u << ((r + 1) / kBwdRows);
+                                }
                             }
                         }
                     }
@@ -387,12 +409,15 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                         int at = 0;
                         if (lane == 0) at = atomicAdd(&slots_n[t], __popc(bal));
                         at = __shfl_sync(FULL, at, 0) + __popc(bal & lt_mask);
-                        if ((bal >> lane) & 1u) sm.slots[FB_IDX(t * 32 * warps + at, q.row_tiles * 32 * warps, p.err)] = (uint8_t)(32 * warp + lane);
+                        if ((bal >> lane) & 1u) {
+                            at = FB_IDX(t * 32 * warps + at, q.row_tiles * 32 * warps, p.err);
+                            sm.slots[at] = (uint8_t)(32 * warp + lane);
+                        }
                     }
                 }
                 __syncthreads();
 
-                // ---- products: 8 cells at a time
+                // ---- products: 16 cells at a time
                 if (!again) {
 #pragma unroll
                     for (int i = 0; i < RT; ++i) {
@@ -403,14 +428,14 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                         const int n_slots = slots_n[row_tile];
 #pragma unroll 1
                         for (int k = 16 * group; k < n_slots; k += 16 * q.groups) {
-                            // (fragments: rows lane / 4 and + 8, cells 2 (lane % 4) and + 1, + 8, + 9.  Cells past the last one: the
-                            // last one, with weight 0)
+                            // (fragments: rows lane / 4 and + 8, cells 2 (lane % 4) and + 1, + 8, + 9.  Cells past the last
+                            // one: the last one, with weight 0)
                             float g[4][NT], w[4][2];
 #pragma unroll
                             for (int c = 0; c < 4; ++c) {
                                 const int at = k + 2 * (lane & 3) + (c & 1) + (c >> 1) * 8, slot = slots[min(at, n_slots - 1)];
-                                const float *const src =
-                                    gout + (size_t)FB_IDX(sm.list[first + slot], p.X * p.Y, p.err) * (unsigned)p.C + ch0 + (lane >> 2);
+                                const size_t cell = FB_IDX(sm.list[first + slot], p.X * p.Y, p.err);
+                                const float *const src = gout + cell * (unsigned)p.C + ch0 + (lane >> 2);
 #pragma unroll
                                 for (int j = 0; j < NT; ++j)
                                     g[c][j] = WHOLE || ch0 + 8 * j + (lane >> 2) < p.C ? __ldg(src + 8 * j) : 0.f;
@@ -425,7 +450,8 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                                 split_bf16(g[0][j], g[1][j], bh[0], bm[0], bl[0]);
                                 split_bf16(g[2][j], g[3][j], bh[1], bm[1], bl[1]);
                                 float t[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f};
-                                // (mid x lo, lo x mid and lo x lo are left out: at most 2^-24 of a product, 2^-27 root mean square)
+                                // (mid x lo, lo x mid and lo x lo are left out: at most 2^-24 of a product, 2^-27 root mean
+                                // square)
                                 mma_bf16(t, ah, bh[0], bh[1]);
                                 mma_bf16(u, ah, bl[0], bl[1]);
                                 mma_bf16(u, al, bh[0], bh[1]);
@@ -446,7 +472,8 @@ __global__ void __launch_bounds__(kBwdMaxWarps * 32, NT * RT <= 4 ? 3 : 2) vt_te
                             if (r / kBwdRows % q.row_warps != row_warp) continue;
                             const float w = sm.weights[r * pitch + c];
                             if (w == 0.f) continue;
-                            for (int ch = ch0 + lane; ch < min(ch0 + 8 * NT, p.C); ch += 32) atomicAdd(dst + (size_t)r * rowf + ch, w * __ldg(src + ch));
+                            for (int ch = ch0 + lane; ch < min(ch0 + 8 * NT, p.C); ch += 32)
+                                atomicAdd(dst + (size_t)r * rowf + ch, w * __ldg(src + ch));
                         }
                     }
                 }

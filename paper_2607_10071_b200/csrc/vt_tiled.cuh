@@ -806,8 +806,8 @@ __global__ void __launch_bounds__(WARPS * 32, (V == 4 ? 12 : FB_WARPS_PER_SM) / 
     // pyramid levels before (LEVEL).  The copy, or the first level, lets this grid start only when its own wait is over, so that
     // whatever ran before the call has completed.  All are no-ops for a launch without the attribute.
     // (pyramid of three 105 -> 96 us, planar 75 -> 71 us, ragged rows 47 -> 44 us: a grid's geometry runs in the tail of the one before.
-    // Instances of their own for pyramid levels take 0.5-1 % off the others, but not of one fp32 vector per lane: there the smallest
-    // calls measure 7.1 us with one instance for both, decided by the parameters, and 7.4 us with two.)
+    // Pyramid levels have instances of their own so that the others carry no choice, which is 0.2-0.8 %, inside the noise of most;
+    // but not of one fp32 vector per lane: there the smallest calls measured 7.1 us with one instance for both and 7.4 us with two.)
     constexpr bool kBoth = ((V == 1 && !BF16) || WARPS != 4) && !PLANAR && !BWD;  // (other CTA sizes are hints: one instance for both)
     const bool adds = kBoth ? p.accumulate != 0 : LEVEL && p.accumulate;
     const bool chained = !BWD && (PLANAR || (kBoth ? adds : LEVEL));
