@@ -1153,8 +1153,9 @@ flashbev_status launch_tiled(const flashbev_vt_params *p, cudaStream_t stream, b
     return e == cudaSuccess ? FLASHBEV_OK : FLASHBEV_CUDA_ERROR;
 }
 
-// Chooses the tiles and the grid of the texel-side backward kernel.  NT: channels per warp / 8; RT: row tiles per warp.
-flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, int &NT, int &RT, dim3 &grid, size_t &smem)
+// Chooses the tiles and the grid of the texel-side backward kernel.  NT: channels per warp / 8; RT: row tiles per warp; pays: whether
+// the CTAs have enough to do.
+flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, int &NT, int &RT, dim3 &grid, size_t &smem, bool &pays)
 {
     q = {};
     q.k = base_params(p);
@@ -1194,6 +1195,13 @@ flashbev_status configure_backward(const flashbev_vt_params *p, BwdParams &q, in
     const double most = std::min({8.0, std::floor(resident / columns), std::floor(cells / std::max(p->N, 5) / 20.0)});
     q.slices = (int)std::max(two ? 2.0 : 1.0, most);
     q.exclusive = q.slices == 1;
+    // A CTA's survey and tables cost the same however few cells reach its column.  One wave of them takes no longer than the scatter,
+    // but with more of them than the SMs hold at once a column needs 30 samples (cells x height bins per column of a camera's map) to
+    // pay for its CTA.  Scatter / texel side, us: C = 80, 8 x 63 x 84 maps, two frames of 28 x 47 x 2 14 / 31; C = 64, 7 x 55 x 144,
+    // 75 x 53 x 4 15 / 20; C = 128, 7 x 49 x 144, 99 x 98 x 2 23 / 36.  Over 440 calls of 2 to 200 samples this line is within 3.5 % of
+    // the better kernel (geometric mean; without it 9 %, at the worst 2.9 times), and behind the texel side by 15 % at the worst.  Not
+    // with up to 40 channels (80 calls: 2.0 % without it, 2.1 % and up to 1.4 times with it).
+    pays = p->C <= 40 || columns * q.slices <= 1.2 * resident || (double)p->X * p->Y * p->Z >= 30.0 * p->N * p->feat_w;
     smem = bwd_smem_layout(nullptr, nullptr, p->N, q.row_tiles, q.row_warps, q.ch_tiles, q.groups, NT, RT, p->reduce);
     const double blocks = (double)p->B * p->N * p->feat_w * q.slices;
     if (blocks > 2147483647.0 || cblocks > 65535 || rblocks > 65535 || smem > 200 * 1024) return FLASHBEV_UNSUPPORTED;
@@ -1221,15 +1229,16 @@ cudaError_t launch_backward(const BwdParams &q, dim3 grid, size_t smem, cudaStre
 // Which of the two backward kernels takes a call: the texel-side one, but not
 // - with hints, which are launch geometry of the scatter;
 // - with more than 64 height bins, each of which it projects (the scatter solves for intervals);
+// - with more columns than the SMs hold at once and too little for each (`pays` above);
 // - with up to 40 channels, unless in SUM mode on few cells: it makes its geometry, and the mean modes their counts, for every texel
 //   column that a cell reaches, whatever the channels.  Scatter / texel side, us in a graph, six tilted cameras, 32 x 88 maps, 8 bins,
 //   6 k, 20 k and 62 k cells: C = 32 SUM 14 / 12, 27 / 28, 57 / 72, mean 14 / 14, 27 / 33, 57 / 89, Eq. 1 14 / 14, 28 / 32, 58 / 82;
 //   C = 16 SUM 13 / 10, 21 / 21, 43 / 53; C = 8 SUM 12 / 10, 18 / 22, 34 / 56.  The line in cells, 50 per texel column, loses a
 //   quarter at the most against the better one of the two (16 x 44 maps, C = 32, SUM: 10 k cells 15 / 18, 20 k 22 / 18).  At C = 40,
 //   where the scatter's lanes divide badly, the texel side would win in all three modes (19 / 10, 37 / 22, 83 / 58 in SUM).
-// Above 40 channels it wins: 54 of 60 drawn calls of 48 to 256 channels, by up to 3.2x (geometric mean 1.50; 200 x 200 x 8, C = 80
-// 87 / 34, C = 128 on tilted cameras, Eq. 1 137 / 88); the others take up to 1.13 times as long, one of them 1.27 times (C = 64,
-// 55 x 144 maps, 75 x 53 x 4 cells: 15 / 19).
+// Otherwise it wins: over 100 drawn calls of 48 to 256 channels by 1.5x (geometric mean, 3.2x at most; 200 x 200 x 8, C = 80 87 / 34,
+// C = 128 on tilted cameras, Eq. 1 137 / 88), and is 1.13 times as slow at the worst (C = 192, two frames of seven 28 x 175 maps,
+// tilted, 137 x 56 x 5: 56 / 63).
 bool backward_by_texel(const flashbev_vt_params *p)
 {
     for (int t : p->tune)
@@ -1238,14 +1247,18 @@ bool backward_by_texel(const flashbev_vt_params *p)
     return p->C > 40 || (p->reduce == FLASHBEV_REDUCE_SUM && (double)p->X * p->Y <= 50.0 * p->N * p->feat_w);
 }
 
-flashbev_status launch_texel_backward(const flashbev_vt_params *p, const float *grad_out, float *grad_features, cudaStream_t stream)
+// (`always`: also where it does not pay)
+flashbev_status launch_texel_backward(const flashbev_vt_params *p, const float *grad_out, float *grad_features, cudaStream_t stream,
+                                      bool always)
 {
     BwdParams q;
     int NT, RT;
     dim3 grid;
     size_t smem;
-    const flashbev_status st = configure_backward(p, q, NT, RT, grid, smem);
+    bool pays;
+    const flashbev_status st = configure_backward(p, q, NT, RT, grid, smem, pays);
     if (st != FLASHBEV_OK) return st;
+    if (!always && !pays) return FLASHBEV_UNSUPPORTED;
     q.k.feat = nullptr, q.k.out = nullptr, q.k.count_out = nullptr;
     q.k.gout = grad_out, q.k.gfeat = grad_features;
     if (!q.exclusive) {
@@ -1492,8 +1505,9 @@ flashbev_status flashbev_sampling_vt_backward(const flashbev_vt_backward_params 
         return FLASHBEV_MISALIGNED;
     if (q->C % 4 || !tiled_applicable(&p)) return FLASHBEV_UNSUPPORTED;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    if (backward_by_texel(&p)) {
-        st = launch_texel_backward(&p, q->grad_out, q->grad_features, stream);
+    const bool texel = backward_by_texel(&p);
+    if (texel) {
+        st = launch_texel_backward(&p, q->grad_out, q->grad_features, stream, false);
         if (st != FLASHBEV_UNSUPPORTED) return st;
     }
     KParams k;
@@ -1509,7 +1523,8 @@ flashbev_status flashbev_sampling_vt_backward(const flashbev_vt_backward_params 
         if (!(p.tune[3] & 0xff0)) p.tune[3] |= (1 << 4) | (2 << 8);
         if (!(p.tune[3] & 0xc0000)) p.tune[3] |= 0x40000;
     }
-    if ((st = configure_tiled(&p, k, V, warps, grid, smem, false, true)) != FLASHBEV_OK) return st;
+    if ((st = configure_tiled(&p, k, V, warps, grid, smem, false, true)) != FLASHBEV_OK)  // (more than 65535 batch elements)
+        return texel && st == FLASHBEV_UNSUPPORTED ? launch_texel_backward(&p, q->grad_out, q->grad_features, stream, true) : st;
     k.feat = nullptr, k.out = nullptr, k.count_out = nullptr;
     k.gout = q->grad_out, k.gfeat = q->grad_features;
     const size_t bytes = (size_t)q->B * q->N * q->feat_h * q->feat_w * q->C * sizeof(float);
