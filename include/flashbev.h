@@ -216,8 +216,9 @@ flashbev_status flashbev_sampling_vt_host_static(const flashbev_vt_params *p, vo
  *
  * Enqueues one kernel on `stream` that takes the sums texel by texel (after a memset of `grad_features` to zero where there are
  * so few texel columns that several blocks share one), or (few channels over many cells, many texel columns over few cells, more
- * than 64 height bins, launch hints in `tune`) a memset and a kernel that scatters with fp32 vector atomics.  The summation order -- and the last bits of the
- * result -- can differ from run to run.  Allocates nothing.  C must be a multiple of 4 and both gradient pointers 16-byte aligned, else FLASHBEV_UNSUPPORTED / FLASHBEV_MISALIGNED.
+ * than 64 height bins, launch hints in `tune`) a memset and a kernel that scatters with fp32 vector atomics.  The summation order
+ * -- and the last bits of the result -- can differ from run to run.  Allocates nothing.  C must be a multiple of 4 and both
+ * gradient pointers 16-byte aligned, else FLASHBEV_UNSUPPORTED / FLASHBEV_MISALIGNED.
  */
 typedef struct flashbev_vt_backward_params {
     size_t struct_size;        /* sizeof(flashbev_vt_backward_params) of the caller's header */
